@@ -72,3 +72,25 @@ def test_bad_grid_is_refused(ctx):
     ha, hb = ctx.load(A), ctx.load(B)
     with pytest.raises(pierce.PierceError):
         pierce.pj_estimate_join(ctx.h, ha, hb, 257)
+
+
+@pytest.mark.parametrize("sides,bands", [(3, 1), (16, 31), (17, 29), (18, 27), (64, 20)])
+def test_volumes_at_the_edges_of_the_triangle_split(ctx, sides, bands):
+    # prisms of 2 sides (bands + 1) triangles (12, 1,024, 1,020, 1,008, 2,688)
+    # around the 1,024 triangles a warp takes, so that meshes end inside, at and
+    # past its range; then boxes as large as the grid (the largest terms) and
+    # triangles turned around, which loading accepts and the sum must follow
+    th = 2 * np.pi * np.arange(sides) / sides
+    meshes = []
+    for k in range(7):
+        r = 3000 + 500 * k
+        foot = np.rint(np.stack([r * np.cos(th), r * np.sin(th)], 1) + 20000 + 30000 * k)
+        meshes.append(synth.building(foot, 1000 * k, 4000, 700, bands))
+    meshes.append(synth.box((0, 0, 0), (262143, 262143, 262143)))
+    v, t = meshes[2]
+    flipped = t.copy()
+    flipped[::3] = flipped[::3][:, [0, 2, 1]]
+    meshes.append((v, flipped))
+    A = synth.concat(meshes)
+    _check(ctx, A, synth.concat(meshes[::-1]), 8)
+    _check(ctx, A, A, 5)
