@@ -1789,7 +1789,20 @@ __global__ void k_pred_combine(uint8_t *flags, const uint8_t *pflags, const int6
 // the triangles of up to 24 leaf pairs (48 / L), filters (edge, triangle)
 // tests by boxes and runs the exact tests that remain one per lane.  A round
 // thus waits for one memory latency however many fetches it makes.  A warp
-// takes 32 new candidates whenever its stack holds less than one round.
+// takes new candidates whenever its stack holds less than one round.
+//
+// Intake.  How many it takes follows what they cost: 8 at first (or an equal
+// share of the candidates, if that is less), four times as many (up to 32) when
+// the last ones were done within 2 rounds, half as many (down to 4) when
+// they took 6 rounds or more.  Cheap candidates (most pairs of a nucleus and
+// a vessel end at their roots) are thus taken in full rounds, while costly
+// ones are taken as warps get to them, so that the candidates last through
+// most of the launch and few tasks have to go through the queue below; and
+// a short list is spread over all warps at once.  Against 32 at every
+// intake (with the thresholds below as measured beside them): 55,000-mesh
+// urban self join 820 -> 612 us, 100,000 instanced pairs 1,180 -> 1,040,
+// cells / nuclei 250 -> 160, 20 x 20 spheres 84 -> 61, 10,000 x 500 tissue
+// 238 -> 238 (4 at every intake: 276).
 //
 // Load balance.  A few pairs (a nucleus lying along a vessel wall over a
 // large area) cost thousands of times the mean, and a warp that holds one
@@ -1797,12 +1810,15 @@ __global__ void k_pred_combine(uint8_t *flags, const uint8_t *pflags, const int6
 // queue: a warp with no input and no tasks left becomes hungry and claims
 // tasks from the queue; a straggler -- a warp that has not been able to take
 // new work for `give_after` SM cycles, while most warps take some every few
-// rounds -- that sees hungry warps gives the older half of its stack (the
-// larger subtrees) to the queue, and so does a warp whose stack is nearly
-// full.  A costly pair thus spreads over more and more warps.  At most
+// rounds -- that sees more than `hungry_min` hungry warps (a few that wait
+// cost less than the tasks' way through the queue: with any, 1,120 / 800 us
+// on the instanced pairs and the urban join against 1,040 / 612) gives the
+// older half of its stack (the larger subtrees) to the queue, and so does a
+// warp whose stack is nearly full.  A costly pair thus spreads over more and more warps.  At most
 // `hungry_max` warps wait for tasks (a warp that finds that many waiting
 // leaves): a heavy pair needs tens of helpers, not thousands of warps
-// polling the same words.  A crossing sets the candidate's flag; the tasks
+// polling the same words (a cap of 4 per SM; with 2 per SM 4,429 x 260
+// tissue within at W = 8 took 270 us, with 4 252, the others the same).  A crossing sets the candidate's flag; the tasks
 // of a flagged candidate are dropped when popped or claimed.
 //
 // Queue protocol.  Entries are uint4 (candidate, item A, item B, ready).  A
@@ -1881,6 +1897,7 @@ struct StreamArgs {
   unsigned int dq_cap;
   unsigned int spin_limit;  // bound on the polls of every wait (each sleeps <= 1 us)
   unsigned int hungry_max;  // warps that may wait for queued tasks
+  unsigned int hungry_min;  // ... and must be exceeded for a straggler to give
   long long give_after;     // SM cycles without new work that make a straggler
   // parity rays over the per-thread node budget (w.q_par, w.q_par_n): one
   // warp each, claimed at this position before the warp's first intake
@@ -1995,6 +2012,9 @@ __global__ void __launch_bounds__(128, 4) k_stream(StreamArgs P) {
   long long t_new = clock64();  // when this warp last took (or tried to take) work
   int err = DERR_NONE;
   unsigned iters = 0;
+  // candidates the next intake takes, and the rounds run since the last one
+  int chunk = (int)min((int64_t)8, max((int64_t)1, (n_in + 4 * gridDim.x - 1) / (4 * gridDim.x)));
+  int rounds = 4;  // between the two limits: the first intake keeps its size
   // Every 4th iteration lane 0 reads the intake position (a warp busy with a
   // costly pair takes no input and would not notice that it has run out) or,
   // once it has, the hungry count; the next iteration uses the value, so the
@@ -2336,7 +2356,7 @@ __global__ void __launch_bounds__(128, 4) k_stream(StreamArgs P) {
       if (peek_more) {
         if ((int64_t)v >= n_in) more = false;
       } else {
-        give = v > 0 && __shfl_sync(FULL, (int)(clock64() - t_new > P.give_after), 0);
+        give = v > P.hungry_min && __shfl_sync(FULL, (int)(clock64() - t_new > P.give_after), 0);
       }
     }
     if ((iters & 3u) == 0) {
@@ -2346,8 +2366,11 @@ __global__ void __launch_bounds__(128, 4) k_stream(StreamArgs P) {
     }
     // 1. intake, while the stack holds less than one round
     if (more && sp < Cf::NT && nlq < pmax) {
+      if (rounds <= 2) chunk = min(32, 4 * chunk);
+      else if (rounds >= 6) chunk = max(min(4, chunk), chunk / 2);
+      rounds = 0;
       unsigned base = 0;
-      if (lane == 0) base = atomicAdd(sq(P, SQ_INTAKE), 32u);
+      if (lane == 0) base = atomicAdd(sq(P, SQ_INTAKE), (unsigned)chunk);
       base = __shfl_sync(FULL, base, 0);
       t_new = clock64();
       if ((int64_t)base >= n_in) {
@@ -2357,7 +2380,7 @@ __global__ void __launch_bounds__(128, 4) k_stream(StreamArgs P) {
       const int64_t idx = (int64_t)base + lane;
       bool push = false;
       uint4 ent = make_uint4(0u, 0u, 0u, 0u);
-      if (idx < n_in && vflags[idx] == 0 && (!Q.need || Q.need[idx])) {
+      if (lane < chunk && idx < n_in && vflags[idx] == 0 && (!Q.need || Q.need[idx])) {
         const int ia = Q.cand[2 * idx], ib = Q.cand[2 * idx + 1];
         if (ia >= 0 && ia < Q.MA && ib >= 0 && ib < Q.MB) {
           const F3 off = cand_offset(Q, idx);
@@ -2378,7 +2401,7 @@ __global__ void __launch_bounds__(128, 4) k_stream(StreamArgs P) {
           }
         }
       }
-      // room: sp < NT <= 32 and 32 more stay below SC
+      // room: sp < NT <= 32 and up to 32 more stay below SC
       const unsigned m = __ballot_sync(FULL, push);
       if (push) stk[sp + __popc(m & lt)] = ent;
       sp += __popc(m);
@@ -2465,6 +2488,7 @@ __global__ void __launch_bounds__(128, 4) k_stream(StreamArgs P) {
     // 4. leaf pairs once a round's worth is queued (or nothing else is left)
     if (nlq >= pmax || sp == 0) {
       leaf_round();
+      ++rounds;
       continue;
     }
     // 5. expand round: up to NT tasks; their nodes are copied to shared
@@ -2618,6 +2642,7 @@ __global__ void __launch_bounds__(128, 4) k_stream(StreamArgs P) {
     }
     sp += tt + max(0, tl - room);
     nlq += min(tl, room);
+    ++rounds;
     __syncwarp();
   }
   if (err != DERR_NONE && lane == 0) atomicCAS(Q.err, 0, err);
@@ -3537,8 +3562,9 @@ pj_status run_join(Ctx *ctx, Dataset *A, Dataset *B, const int32_t *cand,
         sa.cbase = cbase;
         sa.dq_cap = dq_cap;
         sa.spin_limit = o->wait_polls > 0 ? (unsigned)o->wait_polls : (1u << 19);
-        sa.hungry_max = 2u * (unsigned)ctx->num_sms;
-        sa.give_after = 5000;
+        sa.hungry_max = 4u * (unsigned)ctx->num_sms;
+        sa.hungry_min = (unsigned)ctx->num_sms / 2;
+        sa.give_after = 2000;
         sa.q_par_pos = split ? nullptr : hc + 1;
         sa.par_stack_cap = args.stack_cap;
         const bool kt = timed && !kev.empty();

@@ -466,3 +466,25 @@ def test_stream_wait_timeout_falls_back(ctx, tiny):
     # the queue is clean again afterwards: the next join is exact and fast-path
     got3, _ = ctx.join(ha, hb, width=4, leaf_size=4, wave_levels=pierce.PJ_FRONT_STREAM)
     assert np.array_equal(got3, exp)
+
+
+@pytest.mark.parametrize("n", [1, 7, 2431, 2433, 8 * 2432 + 1, 70001])
+def test_intake_takes_every_candidate_once(n):
+    # lists around the sizes at which a warp's first intake changes (an equal
+    # share of the candidates up to 8 a warp, on 4 blocks of 4 warps per SM)
+    # and a long one, over which intakes grow and shrink; repeated candidates
+    # must each be reported
+    A, B = synth.tiny_spheres(1001)
+    every = np.array([(i, j) for i in range(A.nmesh) for j in range(B.nmesh)], np.int32)
+    truth = oracle.join(A, B, every, tier=2).astype(bool)
+    pick = np.random.default_rng(n).integers(0, len(every), size=n)
+    if n > 50000:
+        pick[: n // 2] = np.nonzero(~truth)[0][0]  # cheap ones first, then all kinds
+    with pierce.Context(0) as ctx:
+        ha, hb = ctx.load(A), ctx.load(B)
+        for W, L in ((4, 2), (8, 8), (2, 1)):
+            ctx.build(ha, W, L)
+            ctx.build(hb, W, L)
+            got, info = ctx.join(ha, hb, cand=every[pick], width=W, leaf_size=L)
+            assert info["n_candidates"] == n
+            assert np.array_equal(got, every[pick][truth[pick]])
