@@ -321,12 +321,14 @@ pj_status pj_free_pairs(pj_ctx *ctx, pj_pairs *res);
  *            check failed (a candidate id out of range)
  * Uses each dataset's last-built BVH; the two must have the same width and
  * leaf size (else PJ_ERR_INVALID_ARG, nothing queued).  Runs the FP32 filter
- * with int64 fallback, one warp per pair and plain depth-first traversal.
+ * with int64 fallback in the streaming kernel; if a bounded wait of it runs
+ * out, a launch queued behind it redoes every pair with one warp per pair and
+ * plain depth-first traversal (same result, slower).
  * A candidate id out of range is skipped (its flag stays 0) and makes
  * *d_count -1; the next call clears that state.  Asynchronous: the work is enqueued on cuda_stream (NULL: the
  * context's stream) and the outputs are valid once it has completed.
  * n_cand above 16,777,216 is rejected with PJ_ERR_INVALID_ARG.
- * Scratch: a 65,600-byte array in device global memory, defined at file
+ * Scratch: a 2,163,520-byte array in device global memory, defined at file
  * scope in the library; every GPU that loads the library holds it until the
  * process exits.  The first call on a device looks up the array's device
  * address (make that first call before any stream capture).  All calls on a

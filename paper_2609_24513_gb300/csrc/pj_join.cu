@@ -341,6 +341,9 @@ struct RefineArgs {
   // result goes to pflags and flags keeps the crossing result
   int predicate;
   uint8_t *pflags;
+  // non-null: the launch does nothing unless this word is set (the
+  // allocation-free join's fallback after a failed streaming launch)
+  const int *only_if;
 };
 
 struct Cnt {
@@ -1014,6 +1017,7 @@ template <int W, bool EXACT>
 __global__ void __launch_bounds__(128, 4) k_refine(RefineArgs P) {
   pdl_wait();
   pdl_trigger();
+  if (P.only_if && *P.only_if == 0) return;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int group_flag[4];
   __shared__ long long group_cand[4];
@@ -1893,7 +1897,8 @@ struct StreamArgs {
   WaveArgs w;               // meshes, candidates, flags, counters, error word
   unsigned int *ctl;        // SQ_* words
   uint4 *dq;                // shared task queue (all-zero between launches)
-  int2 *cbase;              // per candidate: first triangle of each mesh
+  int2 *cbase;              // per candidate: first triangle of each mesh (null: read
+                            // from the mesh records in every expand round)
   unsigned int dq_cap;
   unsigned int spin_limit;  // bound on the polls of every wait (each sleeps <= 1 us)
   unsigned int hungry_max;  // warps that may wait for queued tasks
@@ -2022,6 +2027,7 @@ __global__ void __launch_bounds__(128, 4) k_stream(StreamArgs P) {
   unsigned peek = 0;
   bool peeked = false, peek_more = false;
   bool registered = true;  // counted in SQ_ACTIVE
+  bool q_full = false;     // the shared queue took no more
   if (lane == 0) atomicAdd(sq(P, SQ_ACTIVE), 1u);
 
   // The parity rays the per-thread kernel handed over: the longest rays,
@@ -2396,7 +2402,7 @@ __global__ void __launch_bounds__(128, 4) k_stream(StreamArgs P) {
           if (overlap_open(ba, bb)) {  // crossings only (parity runs apart)
             const uint2 t = make_task(ra, ba, rb, bb);
             ent = make_uint4((uint32_t)idx, t.x, t.y, 0u);
-            P.cbase[idx] = make_int2(__float_as_int(ta), __float_as_int(tbs));
+            if (P.cbase) P.cbase[idx] = make_int2(__float_as_int(ta), __float_as_int(tbs));
             push = true;
           }
         }
@@ -2473,18 +2479,10 @@ __global__ void __launch_bounds__(128, 4) k_stream(StreamArgs P) {
     // 3. a straggler and hungry warps: give the older half of the stack
     // (from NT / 2 entries: the costliest candidates end in rounds of fewer
     // than NT tasks, 0.257 against 0.265 ms) and of the leaf queue
-    if (give && sp >= Cf::NT / 2) {
-      if (!give_half(sp / 2)) {
-        err = DERR_QUEUE;
-        break;
-      }
-    }
-    if (give && nlq >= pmax) {
-      if (!give_leaves(nlq / 2)) {
-        err = DERR_QUEUE;
-        break;
-      }
-    }
+    // A full queue only ends the sharing: the warp keeps its work (all later
+    // reservations fail too, so what is published stays a prefix).
+    if (give && !q_full && sp >= Cf::NT / 2) q_full = !give_half(sp / 2);
+    if (give && !q_full && nlq >= pmax) q_full = !give_leaves(nlq / 2);
     // 4. leaf pairs once a round's worth is queued (or nothing else is left)
     if (nlq >= pmax || sp == 0) {
       leaf_round();
@@ -2516,7 +2514,14 @@ __global__ void __launch_bounds__(128, 4) k_stream(StreamArgs P) {
     // the node copies, so that they do not queue behind them
     const uint8_t fl = act ? vflags[t.x] : (uint8_t)1;
     const F3 off = act ? cand_offset(Q, t.x) : zero;
-    const int2 cbv = act ? P.cbase[t.x] : make_int2(0, 0);  // for leaf pairs
+    int2 cbv = make_int2(0, 0);  // for leaf pairs
+    if (P.cbase) {
+      if (act) cbv = P.cbase[t.x];
+    } else if (act) {
+      const int ia = Q.cand[2 * (int64_t)t.x], ib = Q.cand[2 * (int64_t)t.x + 1];
+      cbv = make_int2(__float_as_int(Q.A.mrec[3 * (int64_t)ia + 2].y),
+                      __float_as_int(Q.B.mrec[3 * (int64_t)ib + 2].y));
+    }
     // stage: task i, side s, slot j (of W) at float4 index (i * 2 + s) * RS + 2 j;
     // one lane per (task, side) copies the W child slots of an expanding
     // node, or the one slot of the item's own box.  (Spreading a node's
@@ -3104,6 +3109,16 @@ static StreamKernel pick_stream(int W, bool exact) {
   if (W == 4) return exact ? k_stream<4, true> : k_stream<4, false>;
   return exact ? k_stream<8, true> : k_stream<8, false>;
 }
+typedef void (*PairParityKernel)(RefineArgs, int64_t *);
+static PairParityKernel pick_pair_parity(int W);  // defined with its kernel
+
+// when the streaming launch's warps share work (measured beside the kernel)
+static void stream_limits(const Ctx *ctx, StreamArgs &sa) {
+  sa.hungry_max = 4u * (unsigned)ctx->num_sms;
+  sa.hungry_min = (unsigned)ctx->num_sms / 2;
+  sa.give_after = 2000;
+}
+
 static int stream_smem_per_warp(int W) {
   return W == 2 ? stream_warp_bytes<2>() : (W == 4 ? stream_warp_bytes<4>() : stream_warp_bytes<8>());
 }
@@ -3436,6 +3451,7 @@ pj_status run_join(Ctx *ctx, Dataset *A, Dataset *B, const int32_t *cand,
   args.single = -1;
   args.predicate = pred;
   args.pflags = d_pflags;
+  args.only_if = nullptr;
   const bool per_pair = o->launch_mode == PJ_LAUNCH_PER_PAIR;
   // pass 1 spills a pair after this many traversal steps; pass 2 after more;
   // pass 3 finishes everything
@@ -3562,9 +3578,7 @@ pj_status run_join(Ctx *ctx, Dataset *A, Dataset *B, const int32_t *cand,
         sa.cbase = cbase;
         sa.dq_cap = dq_cap;
         sa.spin_limit = o->wait_polls > 0 ? (unsigned)o->wait_polls : (1u << 19);
-        sa.hungry_max = 4u * (unsigned)ctx->num_sms;
-        sa.hungry_min = (unsigned)ctx->num_sms / 2;
-        sa.give_after = 2000;
+        stream_limits(ctx, sa);
         sa.q_par_pos = split ? nullptr : hc + 1;
         sa.par_stack_cap = args.stack_cap;
         const bool kt = timed && !kev.empty();
@@ -3869,15 +3883,28 @@ pj_status run_join(Ctx *ctx, Dataset *A, Dataset *B, const int32_t *cand,
 // device memory is owned by another allocator or budget (a framework's
 // caching allocator, a pool sized at start-up).  The caller passes device
 // buffers for the candidates, the per-candidate flags, the pairs and the
-// count; the little scratch the kernels need (candidate count, work counter,
-// error words, per-chunk counts and offsets of the compaction) lives in one
-// file-scope device array shared by every call on a device.
+// count; the scratch the kernels need (candidate count, work counters, error
+// words, per-chunk counts and offsets of the compaction, the streaming
+// kernel's control words and task queue: 2.1 MB) lives in one file-scope
+// device array shared by every call on a device.
+//
+// The refinement is the streaming kernel's.  A warp per pair in plain
+// depth-first order, one task a step, left the costliest pair to one warp:
+// 1,501 x 75 tissue meshes took 2,200-7,200 us by seed, 121 us now.
 // ---------------------------------------------------------------------------
 constexpr int64_t kNoAllocMaxChunks = 4096;
 constexpr int64_t kNoAllocMaxCand = kNoAllocMaxChunks * CMP_CHUNK;  // 16,777,216
-// int64 words: [0] candidate count, [1] work counter, [2..3] four int error
-// words, [4..7] unused, then kNoAllocMaxChunks chunk counts and as many offsets
-constexpr size_t kNoAllocScratchWords = 8 + 2 * kNoAllocMaxChunks;
+// the streaming launch's task queue (each entry is used once a launch: a
+// join of 1,501 x 75 tissue meshes puts about 15,000 through it; when it is
+// full the warps keep their work)
+constexpr int64_t kNoAllocQueue = 131072;
+// int64 words: [0] candidate count, [1] work counter of the fallback, [2..3]
+// four int error words, [4] work counter of the parity pass, [5] the
+// streaming launch's error word, [6..7] unused, then kNoAllocMaxChunks chunk
+// counts and as many offsets, the streaming launch's control words, its queue
+constexpr size_t kNoAllocCtl = 8 + 2 * kNoAllocMaxChunks;
+constexpr size_t kNoAllocCtlWords = SQ_WORDS / 2;
+constexpr size_t kNoAllocScratchWords = kNoAllocCtl + kNoAllocCtlWords + 2 * kNoAllocQueue;
 static __device__ __align__(256) int64_t g_noalloc_scratch[kNoAllocScratchWords];
 
 static std::mutex g_noalloc_mu;
@@ -3899,11 +3926,88 @@ static pj_status noalloc_scratch(Ctx *ctx, int64_t **out) {
   return PJ_OK;
 }
 
-__global__ void k_noalloc_begin(int64_t *scr, int64_t n) {
+__global__ void __launch_bounds__(256) k_noalloc_begin(int64_t *scr, int64_t n) {
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (t < kNoAllocCtlWords) scr[kNoAllocCtl + t] = 0;
+  // the queue is all-zero unless the last call's streaming launch failed
+  // (k_pair_parity clears that word)
+  if (scr[5] != 0)
+    for (size_t i = t; i < 2 * (size_t)kNoAllocQueue; i += gridDim.x * (size_t)blockDim.x)
+      scr[kNoAllocCtl + kNoAllocCtlWords + i] = 0;
+  if (t > 0) return;
   scr[0] = n;  // candidate count
   scr[1] = 0;  // work counter
   scr[2] = 0;  // error words
   scr[3] = 0;
+  scr[4] = 0;  // work counter of the parity pass
+}
+
+// Containment of the allocation-free join, before its streaming launch: all
+// flags cleared, then one warp per (candidate, direction) whose
+// representative vertex lies in the other mesh's box; 1 where it is inside.
+// (The per-thread parity kernel of the other joins hands its long rays over
+// through a list sized by the candidates, which this entry point has no room
+// for.)  A warp takes an equal share of a short list, 32 candidates of a long
+// one, and checks the boxes of all of them at once.  A ray whose batched pops
+// outgrow the stack is repeated in plain depth-first order, which fits.
+template <int W>
+__global__ void __launch_bounds__(128, 4) k_pair_parity(RefineArgs P, int64_t *stream_err) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *stream_err = 0;
+  WarpMem sm = carve<W>(smem + (size_t)wib * warp_smem_bytes<W>(P.stack_cap), P.stack_cap);
+  Cnt cnt;
+  for (int i = 0; i < C_WARP_NUM; ++i) cnt.v[i] = 0;
+  const int64_t n = *P.n_cand, nw = 4 * (int64_t)gridDim.x;
+  const int step = (int)min((int64_t)32, max((int64_t)1, (n + 2 * nw - 1) / (2 * nw)));
+  const F3 zero = mkf3(0.f, 0.f, 0.f);
+  for (;;) {
+    unsigned long long w = 0;
+    if (lane == 0) w = atomicAdd(P.work, (unsigned long long)step);
+    const int64_t base = (int64_t)__shfl_sync(FULL, w, 0);
+    if (base >= n) break;
+    const int64_t idx = base + lane;
+    int ia = 0, ib = 0, need = 0;  // need: bit 0 B's vertex in A's box, bit 1 the reverse
+    if (lane < step && idx < n) {
+      P.flags[idx] = 0;
+      ia = P.cand[2 * idx];
+      ib = P.cand[2 * idx + 1];
+      if (ia >= 0 && ia < P.MA && ib >= 0 && ib < P.MB) {
+        const float4 *ra = P.A.mrec + 3 * (int64_t)ia, *rb = P.B.mrec + 3 * (int64_t)ib;
+        const float4 a0 = ra[0], a1 = ra[1], a2 = ra[2], b0 = rb[0], b1 = rb[1], b2 = rb[2];
+        need = (b0.w >= a0.x && b0.w <= a1.x && b1.w >= a0.y && b1.w <= a1.y && b2.x >= a0.z &&
+                b2.x <= a1.z) |
+               (a0.w >= b0.x && a0.w <= b1.x && a1.w >= b0.y && a1.w <= b1.y && a2.x >= b0.z &&
+                a2.x <= b1.z) << 1;
+      }
+    }
+    __syncwarp();  // the flags are cleared before any is set
+    for (unsigned m = __ballot_sync(FULL, need != 0); m; m &= m - 1) {
+      const int l = __ffs(m) - 1;
+      const int i = __shfl_sync(FULL, ia, l), j = __shfl_sync(FULL, ib, l);
+      const int nd = __shfl_sync(FULL, need, l);
+      int r = 0;
+      for (int pop = 32;; pop = 1) {
+        r = 0;
+        if (nd & 1)
+          r = pair_inside<W>(P.B, j, zero, P.A, i, zero, sm, lane, P.stack_cap, pop, cnt);
+        if (r == 0 && (nd & 2))
+          r = pair_inside<W>(P.A, i, zero, P.B, j, zero, sm, lane, P.stack_cap, pop, cnt);
+        if (r >= 0 || pop == 1) break;
+      }
+      if (r < 0 && lane == 0) atomicCAS(P.err, 0, DERR_STACK);
+      if (r == 1 && lane == 0) P.flags[base + l] = 1;
+    }
+  }
+  for (int i = 0; i < C_WARP_NUM; ++i) {
+    unsigned long long v = cnt.v[i];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+    if (lane == 0 && v) atomicAdd(P.counters + i, v);
+  }
+}
+
+static PairParityKernel pick_pair_parity(int W) {
+  return W == 2 ? k_pair_parity<2> : (W == 4 ? k_pair_parity<4> : k_pair_parity<8>);
 }
 
 // one block of SCAN_T threads: exclusive scan of the chunk counts, then the
@@ -3949,10 +4053,13 @@ pj_status run_join_noalloc(Ctx *ctx, Dataset *A, Dataset *B, const int32_t *d_ca
   int64_t *d_n = scr;
   unsigned long long *work = reinterpret_cast<unsigned long long *>(scr + 1);
   int *err = reinterpret_cast<int *>(scr + 2);
+  int *stream_err = reinterpret_cast<int *>(scr + 5);
   int64_t *counts = scr + 8, *offs = scr + 8 + kNoAllocMaxChunks;
 
-  // plain depth-first traversal: its stack bound holds by construction, so
-  // there is no overflow to recover from
+  // The streaming kernel, after the containment rays.  Its failures (a
+  // bounded wait that ran out, a full stack that the queue could not take)
+  // stay on the device: a guarded launch then redoes every pair in plain
+  // depth-first order, whose stack bound holds by construction.
   const int depth = std::max(bA.max_depth, 1) + std::max(bB.max_depth, 1);
   const int stack_cap = 1 + (W * W - 1) * depth + 256;
   const int per_warp = smem_per_warp(W, stack_cap);
@@ -3995,10 +4102,42 @@ pj_status run_join_noalloc(Ctx *ctx, Dataset *A, Dataset *B, const int32_t *d_ca
   args.predicate = PJ_PRED_INTERSECTS;
   args.pflags = nullptr;
 
-  k_noalloc_begin<<<1, 1, 0, s>>>(scr, n);
+  args.only_if = stream_err;
+
+  k_noalloc_begin<<<64, 256, 0, s>>>(scr, n);
   if (n > 0) {
     k_check_cand<<<std::min(blocks_for(n, 256), ctx->num_sms * 8), 256, 0, s>>>(
         d_cand, nullptr, n, A->M, B->M, B->d_aabb, err);
+    const PairParityKernel kp = pick_pair_parity(W);
+    int occ_p = 0;
+    PJ_CK(occupancy(ctx->device, (const void *)kp, threads, smem, &occ_p));
+    RefineArgs pa = args;
+    pa.work = reinterpret_cast<unsigned long long *>(scr + 4);
+    const int64_t most = (n + threads / 32 - 1) / (threads / 32);
+    kp<<<(int)std::min<int64_t>((int64_t)std::max(occ_p, 1) * ctx->num_sms, most), threads, smem, s>>>(
+        pa, scr + 5);
+    const StreamKernel ks = pick_stream(W, false);
+    const int ssmem = 4 * stream_smem_per_warp(W);
+    int occ_s = 0;
+    PJ_CK(occupancy(ctx->device, (const void *)ks, 128, ssmem, &occ_s));
+    StreamArgs sa{};
+    sa.w.A = args.A;
+    sa.w.B = args.B;
+    sa.w.cand = d_cand;
+    sa.w.n_cand = d_n;
+    sa.w.flags = d_flags;
+    sa.w.counters = ctx->d_counters;
+    sa.w.err = stream_err;
+    const int L = A->last_bvh.second;
+    sa.w.lshift = L == 1 ? 0 : (L == 2 ? 1 : (L == 4 ? 2 : 3));
+    sa.w.MA = A->M;
+    sa.w.MB = B->M;
+    sa.ctl = reinterpret_cast<unsigned int *>(scr + kNoAllocCtl);
+    sa.dq = reinterpret_cast<uint4 *>(scr + kNoAllocCtl + kNoAllocCtlWords);
+    sa.dq_cap = (unsigned)kNoAllocQueue;
+    sa.spin_limit = 1u << 19;
+    stream_limits(ctx, sa);
+    PJ_CK(launch_pdl(ks, std::max(1, occ_s) * ctx->num_sms, 128, ssmem, s, sa));
     int64_t blocks = std::min<int64_t>((int64_t)occ * ctx->num_sms, (n * 32 + threads - 1) / threads);
     kern<<<(int)std::max<int64_t>(blocks, 1), threads, smem, s>>>(args);
   }

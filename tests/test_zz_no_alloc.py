@@ -77,6 +77,30 @@ def test_noalloc_join_reports_a_bad_id_then_recovers():
         assert np.array_equal(pairs, cand[exp.astype(bool)])
 
 
+@pytest.mark.parametrize("n", [1, 33, 4865, 70001])
+@pytest.mark.parametrize("W,L", [(2, 1), (4, 2), (8, 8)])
+def test_noalloc_join_over_list_lengths_and_bvh_shapes(n, W, L):
+    # around the shares of its containment pass (two a warp, then 32) and of
+    # the streaming launch; boxes inside one another besides the spheres
+    torch = pytest.importorskip("torch")
+    A, B = synth.tiny_spheres(1001)
+    inner = synth.concat([synth.box((k, k, k), (250000 - k, 240000, 230000)) for k in (10, 500)])
+    A = synth.concat([A.mesh(k) for k in range(A.nmesh)] + [inner.mesh(0), inner.mesh(1)])
+    every = np.array([(i, j) for i in range(A.nmesh) for j in range(B.nmesh)], np.int32)
+    truth = oracle.join(A, B, every, tier=2).astype(bool)
+    assert truth[-B.nmesh:].any()
+    pick = np.random.default_rng(n).integers(0, len(every), size=n)
+    with pierce.Context(0) as ctx:
+        ha, hb = ctx.load(A), ctx.load(B)
+        ctx.build(ha, W, L)
+        ctx.build(hb, W, L)
+        for _ in range(2):
+            k, pairs, flags = _noalloc(ctx, ha, hb, every[pick], torch)
+            assert np.array_equal(flags.astype(bool), truth[pick])
+            assert k == int(truth[pick].sum())
+            assert np.array_equal(pairs, every[pick][truth[pick]])
+
+
 def test_noalloc_join_rejects_too_many_candidates_and_mixed_bvh_shapes():
     torch = pytest.importorskip("torch")
     A, B = synth.tiny_spheres(5, n_a=2, n_b=2)
