@@ -98,3 +98,32 @@ def test_pathology_full(ctx, pathology_truth):
               "%d crossings, %d slots, %d relaunches, %d rechecked"
               % (mat, len(got), st["ms_total"], st["ms_trace"], st["ms_materialize"],
                  st["edges"], st["hits"], st["slots"], st["relaunches"], st["recheck_pairs"]))
+
+
+@pytest.mark.parametrize("sides,bands", [(6, 0), (5, 2), (8, 1), (17, 1), (3, 10), (64, 19)])
+@pytest.mark.parametrize("W,L", [(2, 8), (4, 1), (8, 2)])
+def test_packet_sizes(ctx, sides, bands, W, L):
+    # 12, 30, 32, 68, 66 and 2,560 triangles a mesh: around the 32 of a warp's
+    # packet; five meshes, so that packets hold the ends of several; the last
+    # one's triangles are far larger than the others' whole meshes
+    th = 2 * np.pi * np.arange(sides) / sides
+
+    def prism(x, y, z, r):
+        foot = np.rint(np.stack([r * np.cos(th) + x, r * np.sin(th) + y], 1))
+        return synth.building(foot, z, 9000, 1500, max(1, bands)) if bands else \
+            synth.box((x - r, y - r, z), (x + r, y + r, z + 9000))
+
+    A = synth.concat([prism(50000 + 6000 * k, 50000, 20000, 4000 + 100 * k) for k in range(5)])
+    B = synth.concat([prism(52000 + 7000 * k, 51000 + 900 * k, 21000, 3000) for k in range(4)] +
+                     [synth.box((0, 0, 0), (262143, 262143, 262143))])
+    ha, hb = ctx.load(A), ctx.load(B)
+    for pred in ("intersects", "overlap"):
+        want = _truth(A, B, pred)
+        assert len(want) > 0
+        hits = set()
+        for mat in MATS:
+            got, st = pierce.pj_dataset_join(ctx.h, ha, hb, width=W, leaf_size=L, predicate=pred,
+                                             materialize=mat)
+            assert np.array_equal(got, want), (pred, mat)
+            hits.add(st["hits"])
+        assert len(hits) == 1
