@@ -89,11 +89,19 @@ void *ws_get(Ctx *ctx, const char *name, size_t bytes, pj_status *st) {
     w.ptr = nullptr;
     w.cap = 0;
     e = cudaMallocAsync(&w.ptr, want, ex->stream);
+    if (e == cudaErrorMemoryAllocation) {
+      mem_trim(ctx);
+      e = cudaMallocAsync(&w.ptr, want, ex->stream);
+    }
   } else {
     if (w.ptr) cudaFree(w.ptr);
     w.ptr = nullptr;
     w.cap = 0;
     e = cudaMalloc(&w.ptr, want);
+    if (e == cudaErrorMemoryAllocation) {
+      mem_trim(ctx);
+      e = cudaMalloc(&w.ptr, want);
+    }
   }
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -142,6 +150,10 @@ void *pool_get(Ctx *ctx, size_t bytes, cudaError_t *e) {
   while (cap < bytes) cap *= 2;
   void *p = nullptr;
   *e = cudaMalloc(&p, cap);
+  if (*e == cudaErrorMemoryAllocation) {
+    mem_trim(ctx);
+    *e = cudaMalloc(&p, cap);
+  }
   if (*e != cudaSuccess) {
     cudaGetLastError();
     return nullptr;
@@ -398,45 +410,42 @@ static int nblk(Ctx *ctx, int64_t n, int t = 256) {
   return (int)b;
 }
 
-template <typename T>
-static cudaError_t dalloc(T **p, int64_t n) {
-  return cudaMalloc((void **)p, sizeof(T) * (size_t)(n > 0 ? n : 1));
+cudaError_t mem_get(Ctx *ctx, void **p, size_t bytes, cudaStream_t s) {
+  cudaError_t e = cudaMallocFromPoolAsync(p, std::max<size_t>(bytes, 16), ctx->mem, s);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    *p = nullptr;
+  }
+  return e;
 }
 
-void free_bvh(Bvh &b) {
-  cudaFree(b.d_nodes);
-  cudaFree(b.d_roots);
-  cudaFree(b.d_tri_order);
-  cudaFree(b.d_trirec);
+void mem_put(Ctx *ctx, void *p, cudaStream_t s) {
+  (void)ctx;
+  if (p) cudaFreeAsync(p, s);
+}
+
+void mem_trim(Ctx *ctx) {
+  cudaGetLastError();
+  // buffers given back in its order (a serving thread must not wait on a
+  // stream that an API call may be capturing)
+  if (!t_exec) cudaStreamSynchronize(ctx->stream);
+  cudaMemPoolTrimTo(ctx->mem, 0);
+}
+
+void free_bvh(Ctx *ctx, Bvh &b) {
+  for (void *p : {(void *)b.d_nodes, (void *)b.d_roots, (void *)b.d_tri_order, (void *)b.d_trirec})
+    mem_put(ctx, p, ctx->stream);
   b = Bvh();
 }
 
-void free_dataset(Dataset *d) {
-  for (auto &kv : d->bvhs) free_bvh(kv.second);
-  for (auto &kv : d->dbvhs) free_bvh(kv.second);
-  cudaFree(d->d_xyz);
-  cudaFree(d->d_tris);
-  cudaFree(d->d_voff);
-  cudaFree(d->d_toff);
-  cudaFree(d->d_aabb);
-  cudaFree(d->d_lexorder);
-  cudaFree(d->d_emask);
-  cudaFree(d->d_mrec);
+void free_dataset(Ctx *ctx, Dataset *d) {
+  for (auto &kv : d->bvhs) free_bvh(ctx, kv.second);
+  for (auto &kv : d->dbvhs) free_bvh(ctx, kv.second);
+  for (void *p : {(void *)d->d_xyz, (void *)d->d_tris, (void *)d->d_voff, (void *)d->d_toff,
+                  (void *)d->d_aabb, (void *)d->d_lexorder, (void *)d->d_emask,
+                  (void *)d->d_mrec})
+    mem_put(ctx, p, ctx->stream);
 }
-
-// RAII for temporary device buffers of the load pipeline
-struct Tmp {
-  std::vector<void *> p;
-  ~Tmp() {
-    for (void *q : p) cudaFree(q);
-  }
-  template <typename T>
-  cudaError_t get(T **out, int64_t n) {
-    cudaError_t e = dalloc(out, n);
-    if (e == cudaSuccess) p.push_back(*out);
-    return e;
-  }
-};
 
 pj_status load_impl(Ctx *ctx, const float *xyz, int64_t V,
                            const int32_t *tris, int64_t F, const int64_t *voff,
@@ -462,17 +471,20 @@ pj_status load_impl(Ctx *ctx, const float *xyz, int64_t V,
   d->M = M; d->V = V; d->F = F;
   d->h_voff.assign(voff, voff + M + 1);
   d->h_toff.assign(toff, toff + M + 1);
-  PJ_CK(dalloc(&d->d_xyz, 3 * V));
-  PJ_CK(dalloc(&d->d_tris, 3 * F));
-  PJ_CK(dalloc(&d->d_voff, M + 1));
-  PJ_CK(dalloc(&d->d_toff, M + 1));
-  PJ_CK(dalloc(&d->d_aabb, 6 * M));
-  PJ_CK(dalloc(&d->d_lexorder, V));
-  PJ_CK(dalloc(&d->d_emask, F));
-  PJ_CK(dalloc(&d->d_mrec, 3 * M));
+  auto keep = [&](auto **p, int64_t n) {
+    return mem_get(ctx, (void **)p, sizeof(**p) * (size_t)std::max<int64_t>(n, 1), s);
+  };
+  PJ_CK(keep(&d->d_xyz, 3 * V));
+  PJ_CK(keep(&d->d_tris, 3 * F));
+  PJ_CK(keep(&d->d_voff, M + 1));
+  PJ_CK(keep(&d->d_toff, M + 1));
+  PJ_CK(keep(&d->d_aabb, 6 * M));
+  PJ_CK(keep(&d->d_lexorder, V));
+  PJ_CK(keep(&d->d_emask, F));
+  PJ_CK(keep(&d->d_mrec, 3 * M));
   d->bytes = 12 * V + 12 * F + 16 * (M + 1) + 24 * M + 4 * V + F + 48 * M;
 
-  Tmp tmp;
+  TmpMem tmp(ctx, s);
   int32_t *tris_local = nullptr;
   cudaMemcpyKind k = dev_ptrs ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   PJ_CK(cudaMemcpyAsync(d->d_xyz, xyz, sizeof(float) * 3 * V, k, s));
@@ -639,11 +651,22 @@ pj_status pj_create(const pj_config *cfg, pj_ctx **out) {
   cudaError_t e = cudaSetDevice(ctx->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking);
+  if (e == cudaSuccess) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = ctx->device;
+    e = cudaMemPoolCreate(&ctx->mem, &props);
+    unsigned long long keep = kMemKeep;
+    if (e == cudaSuccess)
+      e = cudaMemPoolSetAttribute(ctx->mem, cudaMemPoolAttrReleaseThreshold, &keep);
+  }
   if (e == cudaSuccess) e = cudaMalloc(&ctx->d_counters, sizeof(unsigned long long) * C_NUM);
   if (e == cudaSuccess) e = cudaMemset(ctx->d_counters, 0, sizeof(unsigned long long) * C_NUM);
   if (e != cudaSuccess || exec_init(ctx, &ctx->main) != PJ_OK) {
     cudaGetLastError();
     exec_free(&ctx->main);
+    if (ctx->mem) cudaMemPoolDestroy(ctx->mem);
     delete ctx;
     return e == cudaErrorMemoryAllocation ? PJ_ERR_NO_MEMORY : PJ_ERR_CUDA;
   }
@@ -659,11 +682,13 @@ pj_status pj_destroy(pj_ctx *h) {
   // work that reads the datasets may sit on any stream of the device (the
   // allocation-free join runs on the caller's), so wait for all of it
   cudaDeviceSynchronize();
-  for (auto &kv : ctx->datasets) free_dataset(kv.second.get());
+  for (auto &kv : ctx->datasets) free_dataset(ctx, kv.second.get());
   for (auto &g : ctx->graphs) cudaGraphExecDestroy(g.second);
   exec_free(&ctx->main);
   pool_release(ctx);
   cudaFree(ctx->d_counters);
+  cudaStreamSynchronize(ctx->stream);  // the datasets' buffers are back
+  cudaMemPoolDestroy(ctx->mem);
   cudaStreamDestroy(ctx->stream);
   delete ctx;
   return PJ_OK;
@@ -690,7 +715,7 @@ pj_status pj_load_meshes(pj_ctx *h, const float *xyz, int64_t n_verts,
                            n_meshes, ptr_is_device, d.get());
   if (st != PJ_OK) {
     cudaStreamSynchronize(ctx->stream);
-    free_dataset(d.get());
+    free_dataset(ctx, d.get());
     return st;
   }
   std::unique_lock<std::shared_mutex> wl(ctx->ds_rw);
@@ -719,7 +744,7 @@ pj_status pj_free_dataset(pj_ctx *h, pj_dataset id) {
   // allocation-free join returns once its work is queued): wait for the
   // whole device, not only the context's stream
   cudaDeviceSynchronize();
-  free_dataset(d);
+  free_dataset(ctx, d);
   ctx->datasets.erase(id);
   for (auto &g : ctx->graphs) cudaGraphExecDestroy(g.second);
   ctx->graphs.clear();

@@ -308,19 +308,6 @@ __global__ void k_init_queue(QEntry *q, int64_t M, const int64_t *toff) {
   }
 }
 
-struct TmpB {
-  std::vector<void *> p;
-  ~TmpB() {
-    for (void *q : p) cudaFree(q);
-  }
-  template <typename T>
-  cudaError_t get(T **out, int64_t n) {
-    cudaError_t e = cudaMalloc((void **)out, sizeof(T) * (size_t)(n > 0 ? n : 1));
-    if (e == cudaSuccess) p.push_back(*out);
-    return e;
-  }
-};
-
 pj_status build_bvh(Ctx *ctx, Dataset *ds, int W, int L, cudaStream_t s) {
   const int64_t M = ds->M, F = ds->F;
   const int64_t n_int = F - M;
@@ -328,7 +315,7 @@ pj_status build_bvh(Ctx *ctx, Dataset *ds, int W, int L, cudaStream_t s) {
     int64_t b = (n + 255) / 256, cap = (int64_t)ctx->num_sms * 32;
     return (int)std::max<int64_t>(1, std::min(b, cap));
   };
-  TmpB tmp;
+  TmpMem tmp(ctx, s);
   Bvh bvh;
   bvh.W = W;
   bvh.L = L;
@@ -338,19 +325,19 @@ pj_status build_bvh(Ctx *ctx, Dataset *ds, int W, int L, cudaStream_t s) {
   PJ_CK(tmp.get(&k0, F));
   PJ_CK(tmp.get(&k1, F));
   PJ_CK(tmp.get(&i0, F));
-  PJ_CK(cudaMalloc(&bvh.d_tri_order, sizeof(int32_t) * (size_t)std::max<int64_t>(F, 1)));
+  PJ_CK(mem_get(ctx, (void **)&bvh.d_tri_order, sizeof(int32_t) * (size_t)std::max<int64_t>(F, 1), s));
   struct Guard {
+    Ctx *ctx;
     Bvh *b;
+    cudaStream_t s;
     bool ok = false;
     ~Guard() {
-      if (!ok) {
-        cudaFree(b->d_nodes);
-        cudaFree(b->d_roots);
-        cudaFree(b->d_tri_order);
-        cudaFree(b->d_trirec);
-      }
+      if (ok) return;
+      for (void *p : {(void *)b->d_nodes, (void *)b->d_roots, (void *)b->d_tri_order,
+                      (void *)b->d_trirec})
+        mem_put(ctx, p, s);
     }
-  } guard{&bvh};
+  } guard{ctx, &bvh, s};
   k_morton<<<nb(F), 256, 0, s>>>(ds->d_xyz, ds->d_tris, F, ds->d_toff, M, ds->d_aabb, k0, i0);
   int mbits = 1;
   while ((1ll << mbits) <= M) ++mbits;
@@ -436,13 +423,13 @@ pj_status build_bvh(Ctx *ctx, Dataset *ds, int W, int L, cudaStream_t s) {
     return fail(ctx, PJ_ERR_INVALID_ARG, "dataset too large for 30-bit BVH slot ids");
   bvh.n_nodes = n_nodes;
   bvh.max_depth = hflag[0];
-  PJ_CK(cudaMalloc(&bvh.d_nodes, sizeof(float) * (size_t)n_nodes * sw));
+  PJ_CK(mem_get(ctx, (void **)&bvh.d_nodes, sizeof(float) * (size_t)n_nodes * sw, s));
   PJ_CK(cudaMemcpyAsync(bvh.d_nodes, nodes_tmp, sizeof(float) * (size_t)n_nodes * sw,
                         cudaMemcpyDeviceToDevice, s));
-  PJ_CK(cudaMalloc(&bvh.d_roots, sizeof(int32_t) * (size_t)M));
+  PJ_CK(mem_get(ctx, (void **)&bvh.d_roots, sizeof(int32_t) * (size_t)M, s));
   k_iota_roots<<<nb(M), 256, 0, s>>>(bvh.d_roots, M);
   // 5. triangle records in leaf order
-  PJ_CK(cudaMalloc(&bvh.d_trirec, sizeof(float4) * 3 * (size_t)std::max<int64_t>(F, 1)));
+  PJ_CK(mem_get(ctx, (void **)&bvh.d_trirec, sizeof(float4) * 3 * (size_t)std::max<int64_t>(F, 1), s));
   k_trirec<<<nb(F), 256, 0, s>>>(ds->d_xyz, ds->d_tris, bvh.d_tri_order, ds->d_emask,
                                  ds->d_toff, M, F, bvh.d_trirec);
   PJ_CK(cudaGetLastError());

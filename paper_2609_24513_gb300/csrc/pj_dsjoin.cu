@@ -554,14 +554,13 @@ static pj_status dataset_bvh(Ctx *ctx, Dataset *ds, int W, int L, cudaStream_t s
       box[3 + d] = std::max(box[3 + d], ds->h_aabb[6 * m + 3 + d]);
     }
   int64_t toff[2] = {0, ds->F};
-  PJ_CK(cudaMalloc(&flat.d_toff, sizeof(toff)));
-  PJ_CK(cudaMalloc(&flat.d_aabb, sizeof(box)));
+  TmpMem tmp(ctx, s);
+  PJ_CK(tmp.get(&flat.d_toff, 2));
+  PJ_CK(tmp.get(&flat.d_aabb, 6));
   PJ_CK(cudaMemcpyAsync(flat.d_toff, toff, sizeof(toff), cudaMemcpyHostToDevice, s));
   PJ_CK(cudaMemcpyAsync(flat.d_aabb, box, sizeof(box), cudaMemcpyHostToDevice, s));
   pj_status st = build_bvh(ctx, &flat, W, L, s);
   cudaStreamSynchronize(s);
-  cudaFree(flat.d_toff);
-  cudaFree(flat.d_aabb);
   if (st != PJ_OK) return st;
   Bvh b = flat.bvhs[{W, L}];
   k_set_owner<<<blocks_for(ds->F, 256), 256, 0, s>>>(b.d_trirec, b.d_tri_order, ds->d_toff, ds->M,

@@ -148,6 +148,43 @@ struct Ctx {
   std::multimap<size_t, void *> hpool;
   std::map<void *, size_t> hpool_cap;
   size_t hpool_bytes = 0;
+  // datasets, their BVHs and the temporary buffers of loading and building
+  // come from a memory pool of the context's own: one dataset takes about 50
+  // allocations, and cudaMalloc / cudaFree at 30-150 us each (the latter also
+  // waits for the device) were half of a load, build and free of 9 M
+  // triangles and three quarters of a tiled join.  Free memory beyond
+  // kMemKeep goes back to the device when the stream is next waited for, the
+  // rest with the context (or when an allocation outside the pool fails).
+  cudaMemPool_t mem = nullptr;
+};
+
+constexpr unsigned long long kMemKeep = 4ull << 30;  // bytes
+
+// a buffer of at least one element from the context's memory pool, in stream
+// order, and its way back: work on it on other streams must be complete
+cudaError_t mem_get(Ctx *c, void **p, size_t bytes, cudaStream_t s);
+void mem_put(Ctx *c, void *p, cudaStream_t s);
+// the pool's free memory back to the device (an allocation elsewhere failed)
+void mem_trim(Ctx *c);
+
+// Temporary buffers of loading and building: back to the pool, in stream
+// order, when they go out of scope.
+struct TmpMem {
+  Ctx *ctx;
+  cudaStream_t s;
+  std::vector<void *> p;
+  TmpMem(Ctx *c, cudaStream_t st) : ctx(c), s(st) {}
+  TmpMem(const TmpMem &) = delete;
+  TmpMem &operator=(const TmpMem &) = delete;
+  ~TmpMem() {
+    for (void *q : p) mem_put(ctx, q, s);
+  }
+  template <typename T>
+  cudaError_t get(T **out, int64_t n) {
+    cudaError_t e = mem_get(ctx, (void **)out, sizeof(T) * (size_t)(n > 0 ? n : 1), s);
+    if (e == cudaSuccess) p.push_back(*out);
+    return e;
+  }
 };
 
 // A device buffer of at least `bytes` from the context's result pool (or a
@@ -196,7 +233,8 @@ enum { DERR_NONE = 0, DERR_STACK = 1, DERR_QUEUE = 2, DERR_OFFSET = 3, DERR_TIME
 
 // build.cu
 pj_status build_bvh(Ctx *ctx, Dataset *ds, int W, int L, cudaStream_t s);
-void free_bvh(Bvh &b);
+// (the device must be done with the BVH / dataset)
+void free_bvh(Ctx *ctx, Bvh &b);
 // tune.cu
 pj_status run_autotune(Ctx *ctx, Dataset *A, Dataset *B, const int32_t *cand, int64_t n_cand,
                        int self_join, const pj_tune_space *space, pj_join_opts *best,
@@ -215,7 +253,7 @@ pj_status run_estimate(Ctx *ctx, Dataset *A, Dataset *B, int G, double *cells_ou
 pj_status load_impl(Ctx *ctx, const float *xyz, int64_t V, const int32_t *tris, int64_t F,
                     const int64_t *voff, const int64_t *toff, int64_t M, int dev_ptrs,
                     Dataset *d);
-void free_dataset(Dataset *d);
+void free_dataset(Ctx *ctx, Dataset *d);
 pj_status run_join_tiled(Ctx *ctx, const pj_host_meshes *A, const pj_host_meshes *B,
                          int self_join, const pj_tiled_opts *o, pj_pairs *out,
                          pj_tiled_stats *stats);

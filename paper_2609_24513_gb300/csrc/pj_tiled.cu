@@ -238,8 +238,8 @@ pj_status run_join_tiled(Ctx *ctx, const pj_host_meshes *Am, const pj_host_meshe
       st = run_join(ctx, DA, DB, nullptr, nullptr, -1, 0, self_join, &jo, ctx->stream, &r);
     }
     cudaStreamSynchronize(ctx->stream);
-    free_dataset(DA);
-    if (!self_join && db) free_dataset(DB);
+    free_dataset(ctx, DA);
+    if (!self_join && db) free_dataset(ctx, DB);
     if (st != PJ_OK) {
       pairs_release(ctx, &r);
       if (n + 1 < todo.size()) next.get();

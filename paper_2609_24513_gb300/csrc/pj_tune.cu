@@ -136,13 +136,15 @@ pj_status run_autotune(Ctx *ctx, Dataset *A, Dataset *B, const int32_t *cand, in
   }
   *table_n = std::min(count, table_cap);
   // free the shapes built here that lost; keep the winner as the default
+  // (work that reads one may sit on a caller's stream)
+  cudaDeviceSynchronize();
   for (Dataset *D : {A, B}) {
     const auto &had = D == A ? had_a : had_b;
     for (auto it = D->bvhs.begin(); it != D->bvhs.end();) {
       const bool keep = had.count(it->first) ||
                         (result == PJ_OK && it->first == std::make_pair((int)win.width, (int)win.leaf_size));
       if (!keep) {
-        free_bvh(it->second);
+        free_bvh(ctx, it->second);
         it = D->bvhs.erase(it);
       } else {
         ++it;

@@ -488,3 +488,24 @@ def test_intake_takes_every_candidate_once(n):
             got, info = ctx.join(ha, hb, cand=every[pick], width=W, leaf_size=L)
             assert info["n_candidates"] == n
             assert np.array_equal(got, every[pick][truth[pick]])
+
+
+def test_datasets_over_reused_memory():
+    # datasets loaded, built and freed in turn take each other's memory back:
+    # every join still equals the oracle's, and a second context beside the
+    # first has a pool of its own
+    sets = [synth.tiny_spheres(seed) for seed in (1001, 1002, 1003)]
+    truth = [oracle.join_all(A, B, tier=2) for A, B in sets]
+    with pierce.Context(0) as one, pierce.Context(0) as two:
+        for k in range(12):
+            A, B = sets[k % 3]
+            ctx = one if k % 4 else two
+            W, L = ((4, 2), (2, 1), (8, 8), (4, 4))[k % 4]
+            ha, hb = ctx.load(A), ctx.load(B, device_tensors=True)
+            ctx.build(ha, W, L)
+            ctx.build(hb, W, L)
+            got, _ = ctx.join(ha, hb)
+            assert np.array_equal(got, truth[k % 3])
+            pierce.pj_free_dataset(ctx.h, ha)
+            if k % 5:
+                pierce.pj_free_dataset(ctx.h, hb)
