@@ -254,37 +254,181 @@ __device__ __forceinline__ int64_t mesh_of(const int64_t *off, int64_t M, int64_
   return lo;
 }
 
-__global__ void k_validate_xyz(const float *xyz, int64_t n, unsigned long long *bad) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    float f = xyz[i];
-    bool ok = (f >= 0.f) && (f < 262144.f) && (f == floorf(f));
-    if (!ok) atomicMin(bad, (unsigned long long)i);
+// sentinel boxes of meshes without vertices, and the start of the minima
+__global__ void k_init_aabb(float *aabb, int64_t M) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 6 * M;
+       i += (int64_t)gridDim.x * blockDim.x)
+    aabb[i] = i % 6 < 3 ? 3e38f : -3e38f;
+}
+
+// The quantisation check and every mesh's closed box in one pass over the
+// vertices, kWarpSpan of them per warp (a block per mesh took 35 us for 15
+// meshes of 13,000 vertices: too few blocks).  Coordinates that pass the check
+// are not negative, so their order is that of their bits, and the sentinels'.
+__global__ void __launch_bounds__(256) k_validate_boxes(const float *xyz, int64_t V,
+                                                        const int64_t *voff, int64_t M,
+                                                        int *aabb, unsigned long long *bad) {
+  const int lane = threadIdx.x & 31;
+  const int64_t w = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5);
+  const int64_t v0 = w * kWarpSpan, v1 = min(v0 + kWarpSpan, V);
+  if (v0 >= v1) return;
+  int64_t m = mesh_of(voff, M, v0);  // meshes may have no vertices
+  for (int64_t f0 = v0; f0 < v1; ++m) {
+    const int64_t f1 = min(voff[m + 1], v1);
+    int lo[3] = {__float_as_int(3e38f), __float_as_int(3e38f), __float_as_int(3e38f)};
+    int hi[3] = {__float_as_int(-3e38f), __float_as_int(-3e38f), __float_as_int(-3e38f)};
+    for (int64_t v = f0 + lane; v < f1; v += 32)
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const float f = xyz[3 * v + d];
+        if (!((f >= 0.f) && (f < 262144.f) && (f == floorf(f))))
+          atomicMin(bad, (unsigned long long)(3 * v + d));
+        // + 0: a negative zero counts as zero
+        const int b = __float_as_int(f + 0.f);
+        lo[d] = min(lo[d], b);
+        hi[d] = max(hi[d], b);
+      }
+    if (f1 > f0) {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const int a = __reduce_min_sync(0xffffffffu, lo[d]), b = __reduce_max_sync(0xffffffffu, hi[d]);
+        if (lane == 0) {
+          atomicMin(aabb + 6 * m + d, a);
+          atomicMax(aabb + 6 * m + 3 + d, b);
+        }
+      }
+      f0 = f1;
+    }
   }
 }
 
-__global__ void k_convert_tris(const int32_t *tris_local, int64_t F,
-                               const int64_t *voff, const int64_t *toff,
-                               int64_t M, int32_t *tris_g,
-                               unsigned long long *bad) {
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < F;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    int64_t m = mesh_of(toff, M, t);
-    int64_t nv = voff[m + 1] - voff[m];
-    int a = tris_local[3 * t], b = tris_local[3 * t + 1], c = tris_local[3 * t + 2];
-    bool ok = a >= 0 && b >= 0 && c >= 0 && a < nv && b < nv && c < nv &&
-              a != b && b != c && a != c;
+// the largest box extent on each axis over all meshes, to ext[0..2]
+__global__ void __launch_bounds__(256) k_max_extent(const float *aabb, int64_t M,
+                                                    unsigned long long *ext) {
+  int e[3] = {0, 0, 0};
+  for (int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; m < M;
+       m += (int64_t)gridDim.x * blockDim.x)
+    for (int d = 0; d < 3; ++d) {
+      const float x = aabb[6 * m + 3 + d] - aabb[6 * m + d];
+      if (x > 0.f && x < 262144.f) e[d] = max(e[d], (int)x);
+    }
+  for (int d = 0; d < 3; ++d) {
+    const int x = __reduce_max_sync(0xffffffffu, e[d]);
+    if ((threadIdx.x & 31) == 0 && x) atomicMax(ext + d, (unsigned long long)x);
+  }
+}
+
+// Global vertex ids of the triangles, their check, and the first step of the
+// unique edges: a half-edge (lo, hi) takes a place in the list of its lower
+// vertex (its rank there; ranks from kMaxRank set *big, see load_impl).
+constexpr unsigned kMaxRank = 255;
+
+__global__ void __launch_bounds__(256) k_convert_tris(const int32_t *tris_local, int64_t F,
+                                                      const int64_t *voff, const int64_t *toff,
+                                                      int64_t M, int32_t *tris_g, unsigned *deg,
+                                                      uint8_t *rank, unsigned long long *bad,
+                                                      unsigned long long *big) {
+  const int lane = threadIdx.x & 31;
+  const int64_t w = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5);
+  const int64_t t0 = w * kWarpSpan, t1 = min(t0 + kWarpSpan, F);
+  if (t0 >= t1) return;
+  int64_t m = warp_mesh_of(toff, M, t0, lane);
+  int64_t end = toff[m + 1], vo = voff[m], nv = voff[m + 1] - vo;
+  for (int64_t t = t0 + lane; t < t1; t += 32) {
+    while (end <= t) {
+      ++m;
+      end = toff[m + 1];
+      vo = voff[m];
+      nv = voff[m + 1] - vo;
+    }
+    int id[3] = {tris_local[3 * t], tris_local[3 * t + 1], tris_local[3 * t + 2]};
+    const bool ok = id[0] >= 0 && id[1] >= 0 && id[2] >= 0 && id[0] < nv && id[1] < nv &&
+                    id[2] < nv && id[0] != id[1] && id[1] != id[2] && id[0] != id[2];
     if (!ok) {
       atomicMin(bad, (unsigned long long)t);
-      a = b = c = 0;
+      id[0] = id[1] = id[2] = 0;
     }
-    tris_g[3 * t] = (int32_t)(voff[m] + a);
-    tris_g[3 * t + 1] = (int32_t)(voff[m] + b);
-    tris_g[3 * t + 2] = (int32_t)(voff[m] + c);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) tris_g[3 * t + k] = (int32_t)(vo + id[k]);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const unsigned r = atomicAdd(deg + vo + min(id[k], id[k == 2 ? 0 : k + 1]), 1u);
+      rank[3 * t + k] = (uint8_t)min(r, kMaxRank);
+      if (r >= kMaxRank) *big = 1ull;
+    }
   }
 }
 
-// one block per mesh: closed bounding box of its vertices
+// the half-edges into their lower vertices' lists: (higher vertex, half-edge)
+__global__ void __launch_bounds__(256) k_edge_lists(const int32_t *tris_g, int64_t F,
+                                                    const unsigned *off, const uint8_t *rank,
+                                                    uint2 *list) {
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < F;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    const unsigned id[3] = {(unsigned)tris_g[3 * t], (unsigned)tris_g[3 * t + 1],
+                            (unsigned)tris_g[3 * t + 2]};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const unsigned a = id[k], b = id[k == 2 ? 0 : k + 1];
+      list[off[min(a, b)] + rank[3 * t + k]] = make_uint2(max(a, b), (unsigned)(3 * t + k));
+    }
+  }
+}
+
+// One entry of a vertex's list: if it is the first with its higher vertex,
+// the edge's half-edges are counted; the one that comes first among the
+// triangles owns the edge, any number but two is an open or shared edge.
+__device__ __forceinline__ bool edge_entry(const uint2 *e, int d, int i, unsigned *emask,
+                                           unsigned long long *bad) {
+  const unsigned hi = e[i].x;
+  unsigned own = 0xffffffffu;
+  int n = 0;
+  for (int j = 0; j < d; ++j) {
+    const uint2 q = e[j];
+    if (q.x != hi) continue;
+    if (j < i) return false;
+    ++n;
+    own = min(own, q.y);
+  }
+  if (n != 2) atomicMin(bad, (unsigned long long)own);
+  const unsigned t = own / 3;
+  atomicOr(emask + (t >> 2), 1u << (8 * (t & 3) + own % 3));
+  return true;
+}
+
+// a thread per vertex; a warp for each of the few with long lists (poles)
+constexpr int kLongList = 24;
+
+__global__ void __launch_bounds__(256) k_edge_match(const uint2 *list, const unsigned *off,
+                                                    int64_t V, unsigned *emask,
+                                                    unsigned long long *n_unique,
+                                                    unsigned long long *bad) {
+  const int lane = threadIdx.x & 31;
+  unsigned long long n = 0;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t v0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; v0 < V; v0 += stride) {
+    const int64_t v = v0 + lane;
+    const unsigned b = v < V ? off[v] : 0u;
+    const int d = v < V ? (int)(off[v + 1] - b) : 0;
+    if (d <= kLongList)
+      for (int i = 0; i < d; ++i) n += edge_entry(list + b, d, i, emask, bad);
+    for (unsigned m = __ballot_sync(0xffffffffu, d > kLongList); m; m &= m - 1) {
+      const int l = __ffs(m) - 1;
+      const unsigned lb = __shfl_sync(0xffffffffu, b, l);
+      const int ld = __shfl_sync(0xffffffffu, d, l);
+      for (int i = lane; i < ld; i += 32) n += edge_entry(list + lb, ld, i, emask, bad);
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+  __shared__ unsigned long long s_n[8];
+  if (lane == 0) s_n[threadIdx.x >> 5] = n;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) n += s_n[w];
+    if (n) atomicAdd(n_unique, n);
+  }
+}
+
 // per-mesh record (see Dataset::d_mrec); runs after the boxes and the
 // lexicographic order exist
 __global__ void k_mesh_rec(const float *aabb, const float *xyz, const int32_t *lexorder,
@@ -304,43 +448,6 @@ __global__ void k_mesh_rec(const float *aabb, const float *xyz, const int32_t *l
     rec[3 * m + 1] = make_float4(b[3], b[4], b[5], y);
     rec[3 * m + 2] = make_float4(z, __int_as_float((int)toff[m]), __int_as_float((int)v0),
                                  __int_as_float((int)nv));
-  }
-}
-
-__global__ void k_mesh_aabb(const float *xyz, const int64_t *voff, int64_t M,
-                            float *aabb) {
-  __shared__ float red[6][32];
-  for (int64_t m = blockIdx.x; m < M; m += gridDim.x) {
-    float lo[3] = {3e38f, 3e38f, 3e38f}, hi[3] = {-3e38f, -3e38f, -3e38f};
-    for (int64_t v = voff[m] + threadIdx.x; v < voff[m + 1]; v += blockDim.x) {
-      for (int d = 0; d < 3; ++d) {
-        float f = xyz[3 * v + d];
-        lo[d] = fminf(lo[d], f);
-        hi[d] = fmaxf(hi[d], f);
-      }
-    }
-    for (int d = 0; d < 3; ++d) {
-      for (int o = 16; o > 0; o >>= 1) {
-        lo[d] = fminf(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], o));
-        hi[d] = fmaxf(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], o));
-      }
-    }
-    int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0)
-      for (int d = 0; d < 3; ++d) { red[d][w] = lo[d]; red[3 + d][w] = hi[d]; }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      int nw = blockDim.x >> 5;
-      for (int d = 0; d < 3; ++d) {
-        float a = l < nw ? red[d][l] : 3e38f, b = l < nw ? red[3 + d][l] : -3e38f;
-        for (int o = 16; o > 0; o >>= 1) {
-          a = fminf(a, __shfl_xor_sync(0xffffffffu, a, o));
-          b = fmaxf(b, __shfl_xor_sync(0xffffffffu, b, o));
-        }
-        if (l == 0) { aabb[6 * m + d] = a; aabb[6 * m + 3 + d] = b; }
-      }
-    }
-    __syncthreads();
   }
 }
 
@@ -373,7 +480,8 @@ __global__ void k_edge_runs(const uint64_t *keys, const uint32_t *vals, int64_t 
     atomicOr(&owner_bits[v / 3], 1u << (v % 3));
     ++local;
   }
-  if (local) atomicAdd(n_unique, local);
+  for (int o = 16; o > 0; o >>= 1) local += __shfl_xor_sync(0xffffffffu, local, o);
+  if ((threadIdx.x & 31) == 0 && local) atomicAdd(n_unique, local);
 }
 
 __global__ void k_pack_u8(const uint32_t *in, uint8_t *out, int64_t n) {
@@ -391,6 +499,27 @@ __global__ void k_lex_keys(const float *xyz, int64_t V, const int64_t *voff,
              z = (uint64_t)xyz[3 * v + 2];
     kxyz[v] = (x << 36) | (y << 18) | z;
     kmesh[v] = (uint32_t)mesh_of(voff, M, v);
+    ids[v] = (int32_t)v;
+  }
+}
+
+// mesh, x, y, z in one key: coordinates from the mesh's box, as many bits as
+// the largest box takes on each axis
+__global__ void __launch_bounds__(256) k_lex_keys_box(const float *xyz, int64_t V,
+                                                      const int64_t *voff, int64_t M,
+                                                      const float *aabb, int bx, int by, int bz,
+                                                      uint64_t *key, int32_t *ids) {
+  const int lane = threadIdx.x & 31;
+  const int64_t w = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5);
+  const int64_t v0 = w * kWarpSpan, v1 = min(v0 + kWarpSpan, V);
+  if (v0 >= v1) return;
+  int64_t m = mesh_of(voff, M, v0);  // meshes may have no vertices
+  for (int64_t v = v0 + lane; v < v1; v += 32) {
+    while (voff[m + 1] <= v) ++m;
+    const float *b = aabb + 6 * m;
+    const uint64_t x = (uint64_t)(xyz[3 * v] - b[0]), y = (uint64_t)(xyz[3 * v + 1] - b[1]),
+                   z = (uint64_t)(xyz[3 * v + 2] - b[2]);
+    key[v] = (((((uint64_t)m << bx) | x) << by | y) << bz) | z;
     ids[v] = (int32_t)v;
   }
 }
@@ -480,7 +609,7 @@ pj_status load_impl(Ctx *ctx, const float *xyz, int64_t V,
   PJ_CK(keep(&d->d_toff, M + 1));
   PJ_CK(keep(&d->d_aabb, 6 * M));
   PJ_CK(keep(&d->d_lexorder, V));
-  PJ_CK(keep(&d->d_emask, F));
+  PJ_CK(keep(&d->d_emask, F + 3));  // written in words
   PJ_CK(keep(&d->d_mrec, 3 * M));
   d->bytes = 12 * V + 12 * F + 16 * (M + 1) + 24 * M + 4 * V + F + 48 * M;
 
@@ -493,16 +622,28 @@ pj_status load_impl(Ctx *ctx, const float *xyz, int64_t V,
   PJ_CK(cudaMemcpyAsync(d->d_voff, voff, sizeof(int64_t) * (M + 1), cudaMemcpyHostToDevice, s));
   PJ_CK(cudaMemcpyAsync(d->d_toff, toff, sizeof(int64_t) * (M + 1), cudaMemcpyHostToDevice, s));
 
-  unsigned long long *d_flags = nullptr;  // [0] bad coord, [1] bad tri, [2] bad edge, [3] n unique
-  PJ_CK(tmp.get(&d_flags, 4));
-  unsigned long long init[4] = {~0ull, ~0ull, ~0ull, 0ull};
+  // [0] bad coord, [1] bad tri, [2] bad edge, [3] n unique, [4] a long list,
+  // [5..7] largest box extents
+  unsigned long long *d_flags = nullptr;
+  PJ_CK(tmp.get(&d_flags, 8));
+  unsigned long long init[8] = {~0ull, ~0ull, ~0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
   PJ_CK(cudaMemcpyAsync(d_flags, init, sizeof(init), cudaMemcpyHostToDevice, s));
 
-  if (V > 0) k_validate_xyz<<<nblk(ctx, 3 * V), 256, 0, s>>>(d->d_xyz, 3 * V, d_flags);
-  k_convert_tris<<<nblk(ctx, F), 256, 0, s>>>(tris_local, F, d->d_voff, d->d_toff, M,
-                                              d->d_tris, d_flags + 1);
+  unsigned *deg, *deg_off;  // per vertex: half-edges whose lower vertex it is
+  uint8_t *rank;
+  PJ_CK(tmp.get(&deg, V + 1));  // (a bad triangle's ids may be one past the end)
+  PJ_CK(tmp.get(&deg_off, V + 1));
+  PJ_CK(tmp.get(&rank, 3 * F));
+  PJ_CK(cudaMemsetAsync(deg, 0, sizeof(unsigned) * (V + 1), s));
+  k_init_aabb<<<nblk(ctx, 6 * M), 256, 0, s>>>(d->d_aabb, M);
+  if (V > 0)
+    k_validate_boxes<<<span_blocks(V), 256, 0, s>>>(d->d_xyz, V, d->d_voff, M,
+                                                    reinterpret_cast<int *>(d->d_aabb), d_flags);
+  k_max_extent<<<std::min(nblk(ctx, M), ctx->num_sms), 256, 0, s>>>(d->d_aabb, M, d_flags + 5);
+  k_convert_tris<<<span_blocks(F), 256, 0, s>>>(tris_local, F, d->d_voff, d->d_toff, M, d->d_tris,
+                                                deg, rank, d_flags + 1, d_flags + 4);
   PJ_CK(cudaGetLastError());
-  unsigned long long hf[4];
+  unsigned long long hf[8];
   PJ_CK(cudaMemcpyAsync(hf, d_flags, sizeof(hf), cudaMemcpyDeviceToHost, s));
   PJ_CK(cudaStreamSynchronize(s));
   if (hf[0] != ~0ull) {
@@ -521,11 +662,29 @@ pj_status load_impl(Ctx *ctx, const float *xyz, int64_t V,
     return fail(ctx, PJ_ERR_NOT_MANIFOLD, buf);
   }
 
-  k_mesh_aabb<<<(int)std::min<int64_t>(M, 65535), 256, 0, s>>>(d->d_xyz, d->d_voff, M, d->d_aabb);
-  PJ_CK(cudaGetLastError());
-
-  // unique edges and the closed-manifold check
-  {
+  // Unique edges and the closed-manifold check.  Half-edges meet in the list
+  // of their lower vertex, about three long: a count (with the conversion
+  // above), a scan, a scatter and a comparison within the lists, each about
+  // one pass over the triangles.  A radix sort of all half-edges by 64-bit
+  // keys made sixteen, and its run count queued a million atomics: 3,050 us
+  // for 11 M triangles, 560 now (conversion included).  Lists are compared entry by entry, so
+  // with a vertex of 255 half-edges or more the sort still does it.
+  if (hf[4] == 0) {
+    uint2 *list;
+    PJ_CK(tmp.get(&list, 3 * F));
+    size_t tb = 0;
+    PJ_CK(cub::DeviceScan::ExclusiveSum(nullptr, tb, deg, deg_off, (int)(V + 1), s));
+    char *tstore;
+    PJ_CK(tmp.get(&tstore, (int64_t)tb));
+    PJ_CK(cub::DeviceScan::ExclusiveSum(tstore, tb, deg, deg_off, (int)(V + 1), s));
+    PJ_CK(cudaMemsetAsync(d->d_emask, 0, (size_t)(F + 3) / 4 * 4, s));
+    k_edge_lists<<<nblk(ctx, F), 256, 0, s>>>(d->d_tris, F, deg_off, rank, list);
+    if (V > 0)
+      k_edge_match<<<nblk(ctx, V), 256, 0, s>>>(list, deg_off, V,
+                                                reinterpret_cast<unsigned *>(d->d_emask),
+                                                d_flags + 3, d_flags + 2);
+    PJ_CK(cudaGetLastError());
+  } else {
     int64_t n = 3 * F;
     uint64_t *k0, *k1;
     uint32_t *v0, *v1, *bits;
@@ -545,29 +704,52 @@ pj_status load_impl(Ctx *ctx, const float *xyz, int64_t V,
     k_pack_u8<<<nblk(ctx, F), 256, 0, s>>>(bits, d->d_emask, F);
     PJ_CK(cudaGetLastError());
   }
-  // per-mesh lexicographic vertex order: stable sort by (x, y, z), then
-  // stable sort by mesh
+  // Per-mesh lexicographic vertex order.  One stable sort where mesh, x, y
+  // and z (from the mesh's box) fit 64 bits, of just those bits: 46 bits, six
+  // passes, on 700 nuclei, against eleven of two sorts (by x, y, z, then by
+  // mesh), which larger datasets of large meshes still take.
+  auto bits = [](unsigned long long x) {
+    int b = 0;
+    while (x >> b) ++b;
+    return b;
+  };
+  const int bx = bits(hf[5]), by = bits(hf[6]), bz = bits(hf[7]);
+  const int mb = bits((unsigned long long)(M - 1));
   if (V > 0) {
     uint64_t *kx, *kx2;
-    uint32_t *km, *km2;
-    int32_t *ids, *ids2;
+    int32_t *ids;
     PJ_CK(tmp.get(&kx, V));
     PJ_CK(tmp.get(&kx2, V));
-    PJ_CK(tmp.get(&km, V));
-    PJ_CK(tmp.get(&km2, V));
     PJ_CK(tmp.get(&ids, V));
-    PJ_CK(tmp.get(&ids2, V));
-    k_lex_keys<<<nblk(ctx, V), 256, 0, s>>>(d->d_xyz, V, d->d_voff, M, kx, km, ids);
     size_t tb = 0;
-    PJ_CK(cub::DeviceRadixSort::SortPairs(nullptr, tb, kx, kx2, ids, ids2, (int)V, 0, 54, s));
-    size_t tb2 = 0;
-    PJ_CK(cub::DeviceRadixSort::SortPairs(nullptr, tb2, km, km2, ids2, d->d_lexorder, (int)V, 0, 32, s));
-    void *tstore;
-    PJ_CK(tmp.get((char **)&tstore, (int64_t)std::max(tb, tb2)));
-    PJ_CK(cub::DeviceRadixSort::SortPairs(tstore, tb, kx, kx2, ids, ids2, (int)V, 0, 54, s));
-    // mesh ids in the xyz-sorted order
-    k_gather_u32<<<nblk(ctx, V), 256, 0, s>>>(km, ids2, km2, V);
-    PJ_CK(cub::DeviceRadixSort::SortPairs(tstore, tb2, km2, km, ids2, d->d_lexorder, (int)V, 0, 32, s));
+    char *tstore;
+    if (mb + bx + by + bz <= 64) {
+      const int end = std::max(1, mb + bx + by + bz);
+      k_lex_keys_box<<<span_blocks(V), 256, 0, s>>>(d->d_xyz, V, d->d_voff, M, d->d_aabb, bx, by,
+                                                    bz, kx, ids);
+      PJ_CK(cub::DeviceRadixSort::SortPairs(nullptr, tb, kx, kx2, ids, d->d_lexorder, (int)V, 0,
+                                            end, s));
+      PJ_CK(tmp.get(&tstore, (int64_t)tb));
+      PJ_CK(cub::DeviceRadixSort::SortPairs(tstore, tb, kx, kx2, ids, d->d_lexorder, (int)V, 0,
+                                            end, s));
+    } else {
+      uint32_t *km, *km2;
+      int32_t *ids2;
+      PJ_CK(tmp.get(&km, V));
+      PJ_CK(tmp.get(&km2, V));
+      PJ_CK(tmp.get(&ids2, V));
+      k_lex_keys<<<nblk(ctx, V), 256, 0, s>>>(d->d_xyz, V, d->d_voff, M, kx, km, ids);
+      size_t tb2 = 0;
+      PJ_CK(cub::DeviceRadixSort::SortPairs(nullptr, tb, kx, kx2, ids, ids2, (int)V, 0, 54, s));
+      PJ_CK(cub::DeviceRadixSort::SortPairs(nullptr, tb2, km, km2, ids2, d->d_lexorder, (int)V, 0,
+                                            mb, s));
+      PJ_CK(tmp.get(&tstore, (int64_t)std::max(tb, tb2)));
+      PJ_CK(cub::DeviceRadixSort::SortPairs(tstore, tb, kx, kx2, ids, ids2, (int)V, 0, 54, s));
+      // mesh ids in the xyz-sorted order
+      k_gather_u32<<<nblk(ctx, V), 256, 0, s>>>(km, ids2, km2, V);
+      PJ_CK(cub::DeviceRadixSort::SortPairs(tstore, tb2, km2, km, ids2, d->d_lexorder, (int)V, 0,
+                                            mb, s));
+    }
     PJ_CK(cudaGetLastError());
   }
   if (M > 0) {

@@ -69,15 +69,7 @@ __global__ void __launch_bounds__(256) k_mesh_volume(VolSide A, VolSide B) {
   const VolSide S = w < A.warps ? A : B;
   if (w >= A.warps) w -= A.warps;
   const int64_t t0 = w * kVolTris, t1 = min(t0 + kVolTris, S.F);
-  // the mesh of t0 (every mesh has triangles): 32 probes a step, so that the
-  // search is two or three loads deep
-  int64_t m = 0;
-  for (int64_t n = S.M; n > 1;) {  // toff[m] <= t0 < toff[m + n]
-    const int64_t step = (n + 31) / 32, at = lane * step;
-    const int c = __popc(__ballot_sync(0xffffffffu, at < n && S.toff[m + at] <= t0));
-    m += (c - 1) * step;
-    n = min(step, n - (c - 1) * step);
-  }
+  int64_t m = warp_mesh_of(S.toff, S.M, t0, lane);
   for (int64_t f0 = t0; f0 < t1; ++m) {
     const int64_t f1 = min(S.toff[m + 1], t1);
     const float *p0 = S.xyz + 3 * S.voff[m];

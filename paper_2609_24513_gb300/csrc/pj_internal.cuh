@@ -277,6 +277,32 @@ pj_status mbb_sweep(Ctx *ctx, const Dataset *A, const Dataset *B, bool self_join
 pj_status scan_i64(Ctx *ctx, const int64_t *d_in, int64_t *d_out, int64_t n,
                    int64_t *d_total, cudaStream_t s);
 
+#ifdef __CUDACC__
+// The mesh of element e0 (off[m] <= e0 < off[m + 1], no empty mesh before the
+// result): 32 probes a step, so that a search among thousands of meshes is
+// two or three loads deep.  All lanes of the warp, the same e0 in each.
+__device__ __forceinline__ int64_t warp_mesh_of(const int64_t *off, int64_t M, int64_t e0,
+                                                int lane) {
+  int64_t m = 0;
+  for (int64_t n = M; n > 1;) {  // off[m] <= e0 < off[m + n]
+    const int64_t step = (n + 31) / 32, at = lane * step;
+    const int c = __popc(__ballot_sync(0xffffffffu, at < n && off[m + at] <= e0));
+    m += (c - 1) * step;
+    n = min(step, n - (c - 1) * step);
+  }
+  return m;
+}
+#endif
+
+// elements a warp takes in the kernels over all triangles or vertices: the
+// first one's mesh is searched for once, each lane then follows the offsets
+constexpr int kWarpSpan = 256;
+
+inline int span_blocks(int64_t n) {  // blocks of 256 threads, a span per warp
+  const int64_t b = (n + kWarpSpan * 8 - 1) / (kWarpSpan * 8);
+  return (int)(b < 1 ? 1 : b);
+}
+
 inline int blocks_for(int64_t n, int t) {
   int64_t b = (n + t - 1) / t;
   if (b < 1) b = 1;

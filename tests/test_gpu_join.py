@@ -509,3 +509,58 @@ def test_datasets_over_reused_memory():
             pierce.pj_free_dataset(ctx.h, ha)
             if k % 5:
                 pierce.pj_free_dataset(ctx.h, hb)
+
+
+def _mesh_data(ds):
+    """Boxes, lexicographically first vertices and edge owners in numpy: an
+    edge is owned by the first of its two half-edges in triangle order."""
+    box, lex, own = [], [], []
+    for k in range(ds.nmesh):
+        v, t = ds.mesh(k)
+        box.append(np.concatenate([v.min(0), v.max(0)]))
+        lex.append(np.lexsort((v[:, 2], v[:, 1], v[:, 0]))[0])
+        e = np.sort(np.stack([t, np.roll(t, -1, 1)], -1).reshape(-1, 2), 1).astype(np.int64)
+        _, first = np.unique(e[:, 0] * len(v) + e[:, 1], return_index=True)
+        bits = np.zeros(len(t), np.uint8)
+        np.bitwise_or.at(bits, first // 3, (1 << (first % 3)).astype(np.uint8))
+        own.append(bits)
+    return np.array(box, np.float32), np.array(lex, np.int32), np.concatenate(own)
+
+
+@pytest.mark.parametrize("sides", [3, 11, 12, 13, 127, 128, 300])
+def test_load_over_vertex_valences(ctx, sides):
+    # cap centres of 3 to 300 neighbours, first or last in their meshes: edge
+    # lists below and above the 24 a thread compares and the 255 beyond which
+    # the half-edges are sorted; meshes around the 256 elements of a warp
+    cyl = [synth.cylinder((9000 * k + 5000, 20000, 30000), 1500 + k, 900, sides) for k in range(9)]
+    flip = [(v[::-1].copy(), (len(v) - 1 - t).astype(np.int32)) for v, t in cyl[:4]]
+    ds = synth.concat(cyl + flip + [synth.box((0, 0, 0), (262143, 262143, 262143))])
+    for dev in (False, True):
+        h = ctx.load(ds, device_tensors=dev)
+        got = pierce.pj_export_mesh_data(ctx.h, h, ds.nmesh, len(ds.tris))
+        for a, b in zip(got, _mesh_data(ds)):
+            assert np.array_equal(a, b)
+        assert pierce.pj_dataset_info_get(ctx.h, h)["n_edges"] == 3 * len(ds.tris) // 2
+        pierce.pj_free_dataset(ctx.h, h)
+    # an edge with four triangles, and an open one, are still named
+    v, t = cyl[0]
+    for bad in (np.concatenate([t, t[:1]]), t[1:]):
+        with pytest.raises(pierce.PierceError, match="mesh 1 is not a closed manifold"):
+            ctx.load(synth.concat([cyl[1], (v, bad)]))
+
+
+@pytest.mark.parametrize("n", [1, 2, 1024, 1025, 3000])
+def test_load_vertex_order_over_mesh_counts(ctx, n):
+    # one mesh spans the grid (54 bits of coordinates): with 1,025 meshes or
+    # more its key no longer fits 64 bits and the order takes two sorts
+    rng = np.random.default_rng(n)
+    meshes = [synth.box((0, 0, 0), (262143, 262143, 262143))]
+    for _ in range(n - 1):
+        p = rng.integers(0, 250000, size=3)
+        meshes.append(synth.box(tuple(p), tuple(p + rng.integers(1, 9000, size=3))))
+    ds = synth.concat(meshes)
+    h = ctx.load(ds)
+    got = pierce.pj_export_mesh_data(ctx.h, h, ds.nmesh, len(ds.tris))
+    for a, b in zip(got, _mesh_data(ds)):
+        assert np.array_equal(a, b)
+    pierce.pj_free_dataset(ctx.h, h)
