@@ -18,15 +18,6 @@
 
 namespace pj {
 
-__device__ __forceinline__ int64_t mesh_of_b(const int64_t *off, int64_t M, int64_t e) {
-  int64_t lo = 0, hi = M - 1;
-  while (lo < hi) {
-    int64_t mid = (lo + hi + 1) >> 1;
-    if (off[mid] <= e) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
 __device__ __forceinline__ uint32_t spread10(uint32_t v) {
   v &= 0x3ffu;
   v = (v | (v << 16)) & 0x030000FFu;
@@ -36,20 +27,30 @@ __device__ __forceinline__ uint32_t spread10(uint32_t v) {
   return v;
 }
 
-__global__ void k_morton(const float *xyz, const int32_t *tris, int64_t F,
-                         const int64_t *toff, int64_t M, const float *aabb,
-                         uint64_t *keys, int32_t *ids) {
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < F;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    int64_t m = mesh_of_b(toff, M, t);
+// Morton keys, kWarpSpan triangles per warp.  The grid cell of a centroid is
+// floor(1024 (c - lo) / ext) in integers (sums of three coordinates, below
+// 2^20): the FP64 quotients this replaces gave the same cells and took most
+// of 1,104 us for 11 M triangles (90 now), with a binary search of
+// the mesh per triangle.
+__global__ void __launch_bounds__(256) k_morton(const float *xyz, const int32_t *tris, int64_t F,
+                                                const int64_t *toff, int64_t M,
+                                                const float *aabb, uint64_t *keys,
+                                                int32_t *ids) {
+  const int lane = threadIdx.x & 31;
+  const int64_t w = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5);
+  const int64_t t0 = w * kWarpSpan, t1 = min(t0 + kWarpSpan, F);
+  if (t0 >= t1) return;
+  int64_t m = warp_mesh_of(toff, M, t0, lane), end = toff[m + 1];
+  for (int64_t t = t0 + lane; t < t1; t += 32) {
+    while (end <= t) end = toff[++m + 1];
+    const int64_t a = tris[3 * t], b = tris[3 * t + 1], c = tris[3 * t + 2];
     uint32_t q[3];
+#pragma unroll
     for (int d = 0; d < 3; ++d) {
-      double c = (double)xyz[3 * tris[3 * t] + d] + xyz[3 * tris[3 * t + 1] + d] +
-                 xyz[3 * tris[3 * t + 2] + d];
-      double lo = 3.0 * aabb[6 * m + d], ext = 3.0 * (aabb[6 * m + 3 + d] - aabb[6 * m + d]);
-      double u = ext > 0 ? (c - lo) / ext : 0.0;
-      int iq = (int)(u * 1024.0);
-      q[d] = (uint32_t)min(max(iq, 0), 1023);
+      const int sum = (int)xyz[3 * a + d] + (int)xyz[3 * b + d] + (int)xyz[3 * c + d];
+      const int lo = 3 * (int)aabb[6 * m + d];
+      const unsigned ext = (unsigned)(3 * (int)aabb[6 * m + 3 + d] - lo);
+      q[d] = ext > 0 ? min(((unsigned)(sum - lo) << 10) / ext, 1023u) : 0u;
     }
     uint32_t code = (spread10(q[0]) << 2) | (spread10(q[1]) << 1) | spread10(q[2]);
     keys[t] = ((uint64_t)m << 30) | code;
@@ -60,14 +61,37 @@ __global__ void k_morton(const float *xyz, const int32_t *tris, int64_t F,
 // binary radix tree node arrays (per dataset, internal nodes of mesh m at
 // [ioff[m], ioff[m] + n_m - 1) with ioff[m] = toff[m] - m)
 struct BinTree {
-  int32_t *left, *right;   // >= 0 local internal index, < 0: leaf -(pos + 1)
-  int32_t *first, *last;   // local sorted range
+  int2 *child;             // >= 0 local internal index, < 0: leaf -(pos + 1)
+  int2 *range;             // first and last local sorted position
   int32_t *par_int;        // parent (global internal) of internal node, -1 root
   int32_t *par_leaf;       // parent (global internal) of sorted leaf, -1 none
-  float *box;              // 6 per internal node
-  float *leaf_box;         // 6 per sorted leaf
+  float2 *box;             // 3 per internal node: (lo x, lo y) (lo z, hi x) (hi y, hi z)
+  float2 *leaf_box;        // 3 per sorted leaf
   int32_t *visits;
 };
+
+struct Box6 {
+  float2 a, b, c;
+};
+__device__ __forceinline__ Box6 ld_box(const float2 *p) {
+  Box6 r;
+  r.a = __ldcg(p);
+  r.b = __ldcg(p + 1);
+  r.c = __ldcg(p + 2);
+  return r;
+}
+__device__ __forceinline__ void st_box(float2 *p, const Box6 &r) {
+  __stcg(p, r.a);
+  __stcg(p + 1, r.b);
+  __stcg(p + 2, r.c);
+}
+__device__ __forceinline__ Box6 join(const Box6 &x, const Box6 &y) {
+  Box6 r;
+  r.a = make_float2(fminf(x.a.x, y.a.x), fminf(x.a.y, y.a.y));
+  r.b = make_float2(fminf(x.b.x, y.b.x), fmaxf(x.b.y, y.b.y));
+  r.c = make_float2(fmaxf(x.c.x, y.c.x), fmaxf(x.c.y, y.c.y));
+  return r;
+}
 
 __device__ __forceinline__ int delta(const uint64_t *keys, int64_t base, int n,
                                      int i, int j) {
@@ -78,12 +102,21 @@ __device__ __forceinline__ int delta(const uint64_t *keys, int64_t base, int n,
   return 32 + __clz((uint32_t)i ^ (uint32_t)j);
 }
 
-__global__ void k_karras(const uint64_t *keys, const int64_t *toff,
-                         const int64_t *ioff, int64_t M, int64_t n_int,
-                         BinTree T) {
-  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n_int;
-       g += (int64_t)gridDim.x * blockDim.x) {
-    int64_t m = mesh_of_b(ioff, M, g);
+// the tree's nodes, one per thread (a chain of dependent key reads each: a
+// span of 256 per warp took 54 us for 0.6 M triangles); *big counts those
+// with more than L triangles
+__global__ void __launch_bounds__(256) k_karras(const uint64_t *keys, const int64_t *toff,
+                                                const int64_t *ioff, int64_t M, int64_t n_int,
+                                                BinTree T, int L, unsigned long long *big) {
+  __shared__ unsigned s_big;
+  if (threadIdx.x == 0) s_big = 0;
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const int64_t g0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane, g = g0 + lane;
+  unsigned nbig = 0;
+  int64_t m = g0 < n_int ? warp_mesh_of(ioff, M, g0, lane) : 0;
+  if (g < n_int) {
+    while (ioff[m + 1] <= g) ++m;
     int64_t base = toff[m];
     int n = (int)(toff[m + 1] - toff[m]);
     int i = (int)(g - ioff[m]);
@@ -120,173 +153,230 @@ __global__ void k_karras(const uint64_t *keys, const int64_t *toff,
       right = gamma + 1;
       T.par_int[ib + gamma + 1] = (int32_t)g;
     }
-    T.left[g] = left;
-    T.right[g] = right;
-    T.first[g] = lo;
-    T.last[g] = hi;
+    T.child[g] = make_int2(left, right);
+    T.range[g] = make_int2(lo, hi);
     if (i == 0) T.par_int[g] = -1;
+    nbig += hi - lo + 1 > L;
   }
+  nbig = __reduce_add_sync(0xffffffffu, nbig);
+  if (lane == 0 && nbig) atomicAdd(&s_big, nbig);
+  __syncthreads();
+  if (threadIdx.x == 0 && s_big) atomicAdd(big, (unsigned long long)s_big);
 }
 
-__global__ void k_leaf_boxes(const float *xyz, const int32_t *tris,
-                             const int32_t *sorted, int64_t F, float *leaf_box) {
+// the sorted triangles: their boxes and their records (the key holds the mesh)
+__global__ void __launch_bounds__(256) k_leaves(const float *xyz, const int32_t *tris,
+                                                const int32_t *sorted, const uint64_t *keys,
+                                                const uint8_t *emask, const int64_t *toff,
+                                                int64_t F, float2 *leaf_box, float4 *rec) {
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < F;
        s += (int64_t)gridDim.x * blockDim.x) {
-    int64_t t = sorted[s];
-    for (int d = 0; d < 3; ++d) {
-      float a = xyz[3 * tris[3 * t] + d], b = xyz[3 * tris[3 * t + 1] + d],
-            c = xyz[3 * tris[3 * t + 2] + d];
-      leaf_box[6 * s + d] = fminf(a, fminf(b, c));
-      leaf_box[6 * s + 3 + d] = fmaxf(a, fmaxf(b, c));
-    }
+    const int64_t t = sorted[s], m = (int64_t)(keys[s] >> 30);
+    const float *a = xyz + 3 * (int64_t)tris[3 * t], *b = xyz + 3 * (int64_t)tris[3 * t + 1],
+                *c = xyz + 3 * (int64_t)tris[3 * t + 2];
+    const float ax = a[0], ay = a[1], az = a[2], bx = b[0], by = b[1], bz = b[2];
+    const float cx = c[0], cy = c[1], cz = c[2];
+    rec[3 * s] = make_float4(ax, ay, az, bx);
+    rec[3 * s + 1] = make_float4(by, bz, cx, cy);
+    rec[3 * s + 2] = make_float4(cz, __int_as_float((int)emask[t]),
+                                 __int_as_float((int)(t - toff[m])), 0.f);
+    leaf_box[3 * s] = make_float2(fminf(ax, fminf(bx, cx)), fminf(ay, fminf(by, cy)));
+    leaf_box[3 * s + 1] = make_float2(fminf(az, fminf(bz, cz)), fmaxf(ax, fmaxf(bx, cx)));
+    leaf_box[3 * s + 2] = make_float2(fmaxf(ay, fmaxf(by, cy)), fmaxf(az, fmaxf(bz, cz)));
   }
 }
 
-// bottom-up union of child boxes; the second thread to reach a node computes
-// it (no waiting: the first one stops)
-__global__ void k_refit(const int64_t *toff, const int64_t *ioff, int64_t M,
-                        int64_t F, BinTree T) {
-  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < F;
-       s += (int64_t)gridDim.x * blockDim.x) {
-    int32_t g = T.par_leaf[s];
-    while (g >= 0) {
-      __threadfence();
-      if (atomicAdd(&T.visits[g], 1) == 0) break;
-      __threadfence();
-      int64_t m = mesh_of_b(ioff, M, g);
-      int64_t base = toff[m], ib = ioff[m];
-      float b[6];
-      for (int c = 0; c < 2; ++c) {
-        int32_t ch = c == 0 ? T.left[g] : T.right[g];
-        const float *src = ch < 0 ? T.leaf_box + 6 * (base + (-ch - 1)) : T.box + 6 * (ib + ch);
-        for (int d = 0; d < 6; ++d) {
-          float v = __ldcg(src + d);
-          if (c == 0) b[d] = v;
-          else b[d] = d < 3 ? fminf(b[d], v) : fmaxf(b[d], v);
-        }
-      }
-      for (int d = 0; d < 6; ++d) __stcg(T.box + 6 * (int64_t)g + d, b[d]);
-      g = T.par_int[g];
-    }
+// Bottom-up union of child boxes; the second thread to reach a node computes
+// it (no waiting: the first one stops).  A block takes kRefitT consecutive
+// leaves.  Nodes whose triangles all lie among them -- all but a few per
+// block -- are met and united in shared memory; only above them do threads
+// meet through global memory.  A node's
+// number is one end of its range, so it is also its place in the block.  The
+// version without blocks, with a binary search of the mesh at every step,
+// took 1,910 us for 11 M triangles, 661 now.
+constexpr int kRefitT = 256;
+
+__global__ void __launch_bounds__(kRefitT) k_refit(const uint64_t *keys, const int64_t *toff,
+                                                   const int64_t *ioff, int64_t F, BinTree T) {
+  __shared__ Box6 s_leaf[kRefitT], s_node[kRefitT];
+  __shared__ int s_visit[kRefitT];
+  const int tid = threadIdx.x;
+  const int64_t b0 = blockIdx.x * (int64_t)kRefitT, s = b0 + tid;
+  const int64_t b1 = min(b0 + kRefitT, F);
+  s_visit[tid] = 0;
+  if (s < F) s_leaf[tid] = ld_box(T.leaf_box + 3 * s);
+  __syncthreads();
+  if (s >= F) return;
+  const int64_t m = (int64_t)(keys[s] >> 30), base = toff[m], ib = ioff[m];
+  const int shift = (int)(base - b0);  // local position + shift: place in the block
+  int32_t g = T.par_leaf[s];
+  while (g >= 0) {
+    const int2 rg = T.range[g];
+    if (base + rg.x < b0 || base + rg.y >= b1) break;
+    const int at = (int)(g - ib) + shift;
+    __threadfence_block();
+    if (atomicAdd(&s_visit[at], 1) == 0) return;
+    __threadfence_block();
+    const int2 ch = T.child[g];
+    const volatile float2 *p0 = reinterpret_cast<volatile float2 *>(
+        ch.x < 0 ? &s_leaf[-ch.x - 1 + shift] : &s_node[ch.x + shift]);
+    const volatile float2 *p1 = reinterpret_cast<volatile float2 *>(
+        ch.y < 0 ? &s_leaf[-ch.y - 1 + shift] : &s_node[ch.y + shift]);
+    Box6 x, y;
+    x.a = make_float2(p0[0].x, p0[0].y);
+    x.b = make_float2(p0[1].x, p0[1].y);
+    x.c = make_float2(p0[2].x, p0[2].y);
+    y.a = make_float2(p1[0].x, p1[0].y);
+    y.b = make_float2(p1[1].x, p1[1].y);
+    y.c = make_float2(p1[2].x, p1[2].y);
+    const Box6 r = join(x, y);
+    s_node[at] = r;
+    st_box(T.box + 3 * (int64_t)g, r);
+    g = T.par_int[g];
+  }
+  while (g >= 0) {
+    // releases this thread's box, acquires the sibling's
+    int seen;
+    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;"
+                 : "=r"(seen) : "l"(T.visits + g) : "memory");
+    if (seen == 0) break;
+    const int2 ch = T.child[g];
+    const Box6 x = ld_box(ch.x < 0 ? T.leaf_box + 3 * (base + (-ch.x - 1)) : T.box + 3 * (ib + ch.x));
+    const Box6 y = ld_box(ch.y < 0 ? T.leaf_box + 3 * (base + (-ch.y - 1)) : T.box + 3 * (ib + ch.y));
+    st_box(T.box + 3 * (int64_t)g, join(x, y));
+    g = T.par_int[g];
   }
 }
 
-__global__ void k_count_big(const int32_t *first, const int32_t *last, int64_t n,
-                            int L, unsigned long long *cnt) {
-  unsigned long long c = 0;
-  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n;
-       g += (int64_t)gridDim.x * blockDim.x)
-    c += (last[g] - first[g] + 1) > L;
-  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  if ((threadIdx.x & 31) == 0 && c) atomicAdd(cnt, c);
-}
-
+// Wide node `id`, to be filled from binary node `bin`: >= 0 local internal,
+// < 0 leaf -(pos + 1).  The entries of one level have consecutive ids.
 struct QEntry {
-  int32_t bin;    // binary ref: >= 0 local internal, < 0 leaf -(pos + 1)
+  int32_t bin;
   int32_t mesh;
-  int32_t wide;   // wide node id to fill
-  int32_t depth;
 };
 
-__global__ void k_collapse(const QEntry *qin, const unsigned int *qin_n,
-                           QEntry *qout, unsigned int *qout_n,
-                           unsigned int *node_ctr, int64_t node_cap,
-                           const int64_t *toff, const int64_t *ioff, BinTree T,
-                           float *nodes, int W, int L, int *max_depth, int *err) {
-  int n = (int)*qin_n;
-  int sw = node_stride_words(W);
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
-    QEntry q = qin[e];
-    int64_t base = toff[q.mesh], ib = ioff[q.mesh];
-    int32_t fr[8];
-    int nf = 0;
-    auto count_of = [&](int32_t r) -> int {
-      return r < 0 ? 1 : (T.last[ib + r] - T.first[ib + r] + 1);
+// One level of the top-down collapse: the entries [start[lv], start[lv] +
+// cnt[lv]) become wide nodes; their inner children get the ids after the
+// level's last, a warp's at a time, and are counted in cnt[lv + 1].  The
+// levels follow each other on the device, several to a host round trip (an
+// empty level returns at once): a host wait and a queue per level, and an
+// atomic per child and entry on single words, took 1,939 us for 11 M
+// triangles, 737 now.
+constexpr int kCollapseBatch = 8;
+
+template <int W>
+__global__ void __launch_bounds__(256) k_collapse(QEntry *q, unsigned *start, unsigned *cnt,
+                                                  int lv, int64_t node_cap, const int64_t *toff,
+                                                  const int64_t *ioff, BinTree T, float *nodes,
+                                                  int L, int *err) {
+  const int64_t e0 = start[lv], next = e0 + cnt[lv];
+  const int64_t n = min(next, node_cap) - e0;  // (the capacity is never passed)
+  if (blockIdx.x == 0 && threadIdx.x == 0) start[lv + 1] = (unsigned)next;
+  const int lane = threadIdx.x & 31;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  // warp-uniform trips: the warp's new nodes are numbered together
+  for (int64_t k0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; k0 < n; k0 += stride) {
+    const bool on = k0 + lane < n;
+    int32_t fr[W];
+    int2 rg[W];  // their ranges
+    int nf = 0, inner = 0;
+    int64_t base = 0, ib = 0;
+    QEntry e{0, 0};
+    auto range_of = [&](int32_t r) {
+      return r < 0 ? make_int2(-r - 1, -r - 1) : T.range[ib + r];
     };
-    auto box_of = [&](int32_t r) -> const float * {
-      return r < 0 ? T.leaf_box + 6 * (base + (-r - 1)) : T.box + 6 * (ib + r);
+    auto box_of = [&](int32_t r) {
+      return r < 0 ? T.leaf_box + 3 * (base + (-r - 1)) : T.box + 3 * (ib + r);
     };
-    if (count_of(q.bin) <= L) {
-      fr[nf++] = q.bin;
-    } else {
-      fr[nf++] = T.left[ib + q.bin];
-      fr[nf++] = T.right[ib + q.bin];
-      while (nf < W) {
-        int best = -1;
-        float best_a = -1.f;
-        for (int k = 0; k < nf; ++k) {
-          if (count_of(fr[k]) <= L) continue;
-          const float *b = box_of(fr[k]);
-          float dx = b[3] - b[0], dy = b[4] - b[1], dz = b[5] - b[2];
-          float a = dx * dy + dy * dz + dz * dx;
-          if (a > best_a) { best_a = a; best = k; }
+    auto area_of = [&](int32_t r) {
+      const Box6 b = ld_box(box_of(r));
+      const float dx = b.b.y - b.a.x, dy = b.c.x - b.a.y, dz = b.c.y - b.b.x;
+      return dx * dy + dy * dz + dz * dx;
+    };
+    if (on) {
+      e = q[e0 + k0 + lane];
+      base = toff[e.mesh];
+      ib = ioff[e.mesh];
+      float area[W];  // of those that may be opened, else -1
+      auto put = [&](int k, int32_t r) {
+        const int2 x = range_of(r);
+        const float a = x.y - x.x + 1 <= L ? -1.f : area_of(r);
+#pragma unroll
+        for (int j = 0; j < W; ++j)
+          if (j == k) {
+            fr[j] = r;
+            rg[j] = x;
+            area[j] = a;
+          }
+      };
+      const int2 er = range_of(e.bin);
+      if (er.y - er.x + 1 <= L) {
+        put(nf++, e.bin);
+      } else {
+        const int2 c = T.child[ib + e.bin];
+        put(nf++, c.x);
+        put(nf++, c.y);
+        while (nf < W) {
+          int best = -1;
+          int32_t br = 0;
+          float best_a = -1.f;
+#pragma unroll
+          for (int k = 0; k < W; ++k)
+            if (k < nf && area[k] > best_a) {
+              best_a = area[k];
+              best = k;
+              br = fr[k];
+            }
+          if (best < 0) break;
+          const int2 c2 = T.child[ib + br];
+          put(best, c2.x);
+          put(nf++, c2.y);
         }
-        if (best < 0) break;
-        int32_t r = fr[best];
-        fr[best] = T.left[ib + r];
-        fr[nf++] = T.right[ib + r];
       }
+#pragma unroll
+      for (int k = 0; k < W; ++k) inner += k < nf && rg[k].y - rg[k].x + 1 > L;
     }
-    float *node = nodes + (int64_t)q.wide * sw;
+    // ids of this lane's inner children
+    int incl = inner;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    const int tot = __shfl_sync(0xffffffffu, incl, 31);
+    unsigned first = 0;
+    if (lane == 0 && tot) first = atomicAdd(cnt + lv + 1, (unsigned)tot);
+    int64_t id = next + __shfl_sync(0xffffffffu, first, 0) + (incl - inner);
+    if (!on) continue;
+    float4 *node = reinterpret_cast<float4 *>(nodes + (e0 + k0 + lane) * node_stride_words(W));
     {
-      const float *b = box_of(q.bin);
-      for (int d = 0; d < 6; ++d) node[d] = b[d];
-      node[6] = 0.f;
-      node[7] = 0.f;
+      const Box6 b = ld_box(box_of(e.bin));
+      node[0] = make_float4(b.a.x, b.a.y, b.b.x, b.b.y);
+      node[1] = make_float4(b.c.x, b.c.y, 0.f, 0.f);
     }
+#pragma unroll
     for (int k = 0; k < W; ++k) {
-      float *slot = node + 8 * (k + 1);
-      uint32_t *child = reinterpret_cast<uint32_t *>(slot + 6);
-      slot[7] = 0.f;
       if (k >= nf) {
-        for (int d = 0; d < 3; ++d) {
-          slot[d] = 3e38f;
-          slot[3 + d] = -3e38f;
-        }
-        *child = kEmpty;
+        node[2 * k + 2] = make_float4(3e38f, 3e38f, 3e38f, -3e38f);
+        node[2 * k + 3] = make_float4(-3e38f, -3e38f, __uint_as_float(kEmpty), 0.f);
         continue;
       }
-      int32_t r = fr[k];
-      const float *b = box_of(r);
-      for (int d = 0; d < 6; ++d) slot[d] = b[d];
-      int c = count_of(r);
+      uint32_t word;
+      const int c = rg[k].y - rg[k].x + 1;
       if (c <= L) {
-        int first = r < 0 ? (-r - 1) : T.first[ib + r];
-        *child = kLeafBit | ((uint32_t)first << 3) | (uint32_t)(c - 1);
+        word = kLeafBit | ((uint32_t)rg[k].x << 3) | (uint32_t)(c - 1);
+      } else if (id >= node_cap) {
+        atomicExch(err, 1);
+        word = kEmpty;
+        ++id;
       } else {
-        unsigned int id = atomicAdd(node_ctr, 1u);
-        if ((int64_t)id >= node_cap) {
-          atomicExch(err, 1);
-          *child = kEmpty;
-          continue;
-        }
-        *child = id;
-        unsigned int qs = atomicAdd(qout_n, 1u);
-        QEntry o;
-        o.bin = r;
-        o.mesh = q.mesh;
-        o.wide = (int32_t)id;
-        o.depth = q.depth + 1;
-        qout[qs] = o;
+        word = (uint32_t)id;
+        q[id] = QEntry{fr[k], e.mesh};
+        ++id;
       }
+      const Box6 b = ld_box(box_of(fr[k]));
+      node[2 * k + 2] = make_float4(b.a.x, b.a.y, b.b.x, b.b.y);
+      node[2 * k + 3] = make_float4(b.c.x, b.c.y, __uint_as_float(word), 0.f);
     }
-    atomicMax(max_depth, q.depth);
-  }
-}
-
-__global__ void k_trirec(const float *xyz, const int32_t *tris, const int32_t *sorted,
-                         const uint8_t *emask, const int64_t *toff, int64_t M,
-                         int64_t F, float4 *rec) {
-  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < F;
-       s += (int64_t)gridDim.x * blockDim.x) {
-    int64_t t = sorted[s];
-    int64_t m = mesh_of_b(toff, M, t);
-    const float *a = xyz + 3 * tris[3 * t], *b = xyz + 3 * tris[3 * t + 1],
-                *c = xyz + 3 * tris[3 * t + 2];
-    rec[3 * s] = make_float4(a[0], a[1], a[2], b[0]);
-    rec[3 * s + 1] = make_float4(b[1], b[2], c[0], c[1]);
-    rec[3 * s + 2] = make_float4(c[2], __int_as_float((int)emask[t]),
-                                 __int_as_float((int)(t - toff[m])), 0.f);
   }
 }
 
@@ -296,15 +386,14 @@ __global__ void k_iota_roots(int32_t *roots, int64_t M) {
     roots[m] = (int32_t)m;
 }
 
-__global__ void k_init_queue(QEntry *q, int64_t M, const int64_t *toff) {
+__global__ void k_init_queue(QEntry *q, int64_t M, const int64_t *toff, unsigned *start,
+                             unsigned *cnt) {
   for (int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; m < M;
-       m += (int64_t)gridDim.x * blockDim.x) {
-    QEntry e;
-    e.mesh = (int32_t)m;
-    e.wide = (int32_t)m;
-    e.depth = 1;
-    e.bin = (toff[m + 1] - toff[m] > 1) ? 0 : -1;  // internal 0 is the root
-    q[m] = e;
+       m += (int64_t)gridDim.x * blockDim.x)
+    q[m] = QEntry{(toff[m + 1] - toff[m] > 1) ? 0 : -1, (int32_t)m};  // internal 0 is the root
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    start[0] = 0;
+    cnt[0] = (unsigned)M;
   }
 }
 
@@ -338,7 +427,7 @@ pj_status build_bvh(Ctx *ctx, Dataset *ds, int W, int L, cudaStream_t s) {
         mem_put(ctx, p, s);
     }
   } guard{ctx, &bvh, s};
-  k_morton<<<nb(F), 256, 0, s>>>(ds->d_xyz, ds->d_tris, F, ds->d_toff, M, ds->d_aabb, k0, i0);
+  k_morton<<<span_blocks(F), 256, 0, s>>>(ds->d_xyz, ds->d_tris, F, ds->d_toff, M, ds->d_aabb, k0, i0);
   int mbits = 1;
   while ((1ll << mbits) <= M) ++mbits;
   size_t tb = 0;
@@ -356,28 +445,29 @@ pj_status build_bvh(Ctx *ctx, Dataset *ds, int W, int L, cudaStream_t s) {
   PJ_CK(cudaMemcpyAsync(d_ioff, h_ioff.data(), sizeof(int64_t) * (M + 1),
                         cudaMemcpyHostToDevice, s));
   BinTree T;
-  PJ_CK(tmp.get(&T.left, n_int));
-  PJ_CK(tmp.get(&T.right, n_int));
-  PJ_CK(tmp.get(&T.first, n_int));
-  PJ_CK(tmp.get(&T.last, n_int));
+  PJ_CK(tmp.get(&T.child, n_int));
+  PJ_CK(tmp.get(&T.range, n_int));
   PJ_CK(tmp.get(&T.par_int, n_int));
   PJ_CK(tmp.get(&T.par_leaf, F));
-  PJ_CK(tmp.get(&T.box, 6 * n_int));
-  PJ_CK(tmp.get(&T.leaf_box, 6 * F));
+  PJ_CK(tmp.get(&T.box, 3 * n_int));
+  PJ_CK(tmp.get(&T.leaf_box, 3 * F));
   PJ_CK(tmp.get(&T.visits, n_int));
+  unsigned long long *d_big;  // binary nodes with more than L triangles
+  PJ_CK(tmp.get(&d_big, 1));
+  PJ_CK(cudaMemsetAsync(d_big, 0, 8, s));
   PJ_CK(cudaMemsetAsync(T.par_leaf, 0xff, sizeof(int32_t) * F, s));
   PJ_CK(cudaMemsetAsync(T.visits, 0, sizeof(int32_t) * std::max<int64_t>(n_int, 1), s));
   if (n_int > 0)
-    k_karras<<<nb(n_int), 256, 0, s>>>(k1, ds->d_toff, d_ioff, M, n_int, T);
-  k_leaf_boxes<<<nb(F), 256, 0, s>>>(ds->d_xyz, ds->d_tris, bvh.d_tri_order, F, T.leaf_box);
+    k_karras<<<blocks_for(n_int, 256), 256, 0, s>>>(k1, ds->d_toff, d_ioff, M, n_int, T, L, d_big);
+  // triangle boxes and records in leaf order
+  PJ_CK(mem_get(ctx, (void **)&bvh.d_trirec, sizeof(float4) * 3 * (size_t)std::max<int64_t>(F, 1), s));
+  k_leaves<<<nb(F), 256, 0, s>>>(ds->d_xyz, ds->d_tris, bvh.d_tri_order, k1, ds->d_emask,
+                                 ds->d_toff, F, T.leaf_box, bvh.d_trirec);
   // 3. exact boxes bottom-up
-  if (n_int > 0) k_refit<<<nb(F), 256, 0, s>>>(ds->d_toff, d_ioff, M, F, T);
+  if (n_int > 0)
+    k_refit<<<blocks_for(F, kRefitT), kRefitT, 0, s>>>(k1, ds->d_toff, d_ioff, F, T);
   PJ_CK(cudaGetLastError());
   // 4. collapse to W-wide nodes
-  unsigned long long *d_big;
-  PJ_CK(tmp.get(&d_big, 1));
-  PJ_CK(cudaMemsetAsync(d_big, 0, 8, s));
-  if (n_int > 0) k_count_big<<<nb(n_int), 256, 0, s>>>(T.first, T.last, n_int, L, d_big);
   unsigned long long big = 0;
   PJ_CK(cudaMemcpyAsync(&big, d_big, 8, cudaMemcpyDeviceToHost, s));
   PJ_CK(cudaStreamSynchronize(s));
@@ -385,53 +475,49 @@ pj_status build_bvh(Ctx *ctx, Dataset *ds, int W, int L, cudaStream_t s) {
   const int sw = node_stride_words(W);
   float *nodes_tmp;
   PJ_CK(tmp.get(&nodes_tmp, node_cap * sw));
-  QEntry *qa, *qb;
-  PJ_CK(tmp.get(&qa, node_cap));
-  PJ_CK(tmp.get(&qb, node_cap));
-  unsigned int *ctr;  // [0] qa count, [1] qb count, [2] node counter
-  int *dflag;         // [0] max depth, [1] error
-  PJ_CK(tmp.get(&ctr, 4));
-  PJ_CK(tmp.get(&dflag, 2));
-  unsigned int init[4] = {(unsigned int)M, 0u, (unsigned int)M, 0u};
-  PJ_CK(cudaMemcpyAsync(ctr, init, sizeof(init), cudaMemcpyHostToDevice, s));
-  PJ_CK(cudaMemsetAsync(dflag, 0, 8, s));
-  k_init_queue<<<nb(M), 256, 0, s>>>(qa, M, ds->d_toff);
-  int64_t pending = M;
-  int level = 0;
-  unsigned int *qin_n = ctr, *qout_n = ctr + 1;
-  while (pending > 0) {
-    PJ_CK(cudaMemsetAsync(qout_n, 0, 4, s));
-    k_collapse<<<nb(pending), 256, 0, s>>>(qa, qin_n, qb, qout_n, ctr + 2, node_cap,
-                                          ds->d_toff, d_ioff, T, nodes_tmp, W, L, dflag,
-                                          dflag + 1);
+  QEntry *q;
+  PJ_CK(tmp.get(&q, node_cap));
+  constexpr int kMaxLevels = 4096;
+  unsigned *lvl;  // first entry and number of entries of each level
+  int *dflag;     // node capacity exceeded
+  PJ_CK(tmp.get(&lvl, 2 * (kMaxLevels + 1)));
+  PJ_CK(tmp.get(&dflag, 1));
+  unsigned *start = lvl, *cnt = lvl + kMaxLevels + 1;
+  PJ_CK(cudaMemsetAsync(lvl, 0, sizeof(unsigned) * 2 * (kMaxLevels + 1), s));
+  PJ_CK(cudaMemsetAsync(dflag, 0, 4, s));
+  k_init_queue<<<nb(M), 256, 0, s>>>(q, M, ds->d_toff, start, cnt);
+  const auto kc = W == 2 ? k_collapse<2> : (W == 4 ? k_collapse<4> : k_collapse<8>);
+  const int cgrid = (int)std::min<int64_t>(nb(node_cap), (int64_t)ctx->num_sms * 8);
+  int levels = 0;  // levels with nodes
+  int64_t n_nodes = 0;
+  for (int lv = 0;;) {
+    if (lv + kCollapseBatch > kMaxLevels)
+      return fail(ctx, PJ_ERR_INTERNAL, "BVH collapse did not terminate");
+    for (int k = 0; k < kCollapseBatch; ++k, ++lv)
+      kc<<<cgrid, 256, 0, s>>>(q, start, cnt, lv, node_cap, ds->d_toff, d_ioff, T, nodes_tmp, L,
+                               dflag);
     PJ_CK(cudaGetLastError());
-    unsigned int nxt = 0;
-    PJ_CK(cudaMemcpyAsync(&nxt, qout_n, 4, cudaMemcpyDeviceToHost, s));
+    unsigned h[kCollapseBatch + 1];  // the levels after the batch's first
+    PJ_CK(cudaMemcpyAsync(h, cnt + lv - kCollapseBatch, sizeof(h), cudaMemcpyDeviceToHost, s));
+    int over = 0;
+    PJ_CK(cudaMemcpyAsync(&over, dflag, 4, cudaMemcpyDeviceToHost, s));
     PJ_CK(cudaStreamSynchronize(s));
-    pending = nxt;
-    std::swap(qa, qb);
-    std::swap(qin_n, qout_n);
-    if (++level > 4096) return fail(ctx, PJ_ERR_INTERNAL, "BVH collapse did not terminate");
+    if (over) return fail(ctx, PJ_ERR_INTERNAL, "BVH node capacity exceeded");
+    for (int k = 0; k < kCollapseBatch && h[k]; ++k) {
+      n_nodes += h[k];
+      ++levels;
+    }
+    if (h[kCollapseBatch] == 0) break;
   }
-  unsigned int n_nodes = 0;
-  int hflag[2];
-  PJ_CK(cudaMemcpyAsync(&n_nodes, ctr + 2, 4, cudaMemcpyDeviceToHost, s));
-  PJ_CK(cudaMemcpyAsync(hflag, dflag, 8, cudaMemcpyDeviceToHost, s));
-  PJ_CK(cudaStreamSynchronize(s));
-  if (hflag[1]) return fail(ctx, PJ_ERR_INTERNAL, "BVH node capacity exceeded");
-  if ((int64_t)n_nodes * W >= (1ll << 30))
+  if (n_nodes * W >= (1ll << 30))
     return fail(ctx, PJ_ERR_INVALID_ARG, "dataset too large for 30-bit BVH slot ids");
   bvh.n_nodes = n_nodes;
-  bvh.max_depth = hflag[0];
+  bvh.max_depth = levels;
   PJ_CK(mem_get(ctx, (void **)&bvh.d_nodes, sizeof(float) * (size_t)n_nodes * sw, s));
   PJ_CK(cudaMemcpyAsync(bvh.d_nodes, nodes_tmp, sizeof(float) * (size_t)n_nodes * sw,
                         cudaMemcpyDeviceToDevice, s));
   PJ_CK(mem_get(ctx, (void **)&bvh.d_roots, sizeof(int32_t) * (size_t)M, s));
   k_iota_roots<<<nb(M), 256, 0, s>>>(bvh.d_roots, M);
-  // 5. triangle records in leaf order
-  PJ_CK(mem_get(ctx, (void **)&bvh.d_trirec, sizeof(float4) * 3 * (size_t)std::max<int64_t>(F, 1), s));
-  k_trirec<<<nb(F), 256, 0, s>>>(ds->d_xyz, ds->d_tris, bvh.d_tri_order, ds->d_emask,
-                                 ds->d_toff, M, F, bvh.d_trirec);
   PJ_CK(cudaGetLastError());
   PJ_CK(cudaStreamSynchronize(s));
   bvh.bytes = (int64_t)n_nodes * sw * 4 + 4 * M + 4 * F + 48 * F;

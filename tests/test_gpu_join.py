@@ -564,3 +564,53 @@ def test_load_vertex_order_over_mesh_counts(ctx, n):
     for a, b in zip(got, _mesh_data(ds)):
         assert np.array_equal(a, b)
     pierce.pj_free_dataset(ctx.h, h)
+
+
+@pytest.mark.parametrize("W,L", [(2, 1), (4, 2), (8, 8)])
+def test_bvh_over_block_edges(ctx, W, L):
+    # meshes of 4 to 2,688 triangles, so that trees lie within one of the
+    # refit's blocks of 256 leaves, across two, and over many, and warps'
+    # spans of 256 hold the ends of several meshes
+    th = lambda n: 2 * np.pi * np.arange(n) / n
+    ring = lambda n, r: np.rint(np.stack([r * np.cos(th(n)), r * np.sin(th(n))], 1))
+    meshes = [synth.tetra((9, 9, 9), (90, 9, 9), (9, 90, 9), (9, 9, 90))]
+    for k, (n, b) in enumerate([(3, 1), (16, 7), (17, 7), (4, 31), (64, 20), (3, 1), (5, 50)]):
+        meshes.append(synth.building(ring(n, 4000) + 9000 * (k + 1), 1000 * k, 7000, 900, b))
+        meshes.append(meshes[0])
+    ds = synth.concat(meshes)
+    h = ctx.load(ds)
+    ctx.build(h, W, L)
+    nodes, roots, order = pierce.pj_export_bvh(ctx.h, h, W, L, len(ds.tris), ds.nmesh)
+    box = nodes.view(np.float32)
+    depth = 0
+    for m in range(ds.nmesh):
+        v, t = ds.mesh(m)
+        tri = v[t[order[ds.toff[m]:ds.toff[m + 1]]]]           # in leaf order
+        assert sorted(order[ds.toff[m]:ds.toff[m + 1]]) == list(range(len(t)))
+        seen = np.zeros(len(t), int)
+
+        def walk(n, level):
+            nonlocal depth
+            depth = max(depth, level)
+            lo, hi = np.full(3, 1e9), np.full(3, -1e9)
+            for k in range(1, W + 1):
+                w = int(nodes[n, k, 6]) & 0xFFFFFFFF
+                if w == 0xFFFFFFFF:
+                    continue
+                if w >> 31:
+                    f, c = (w >> 3) & 0x0FFFFFFF, (w & 7) + 1
+                    assert c <= L
+                    seen[f:f + c] += 1
+                    a, b = tri[f:f + c].min((0, 1)), tri[f:f + c].max((0, 1))
+                else:
+                    a, b = walk(w, level + 1)
+                assert np.array_equal(box[n, k, :3], a) and np.array_equal(box[n, k, 3:6], b)
+                lo, hi = np.minimum(lo, a), np.maximum(hi, b)
+            assert np.array_equal(box[n, 0, :3], lo) and np.array_equal(box[n, 0, 3:6], hi)
+            return lo, hi
+
+        walk(int(roots[m]), 1)
+        assert np.all(seen == 1)
+    info = pierce.pj_dataset_info_get(ctx.h, h)
+    assert info["bvh_max_depth"] == depth and info["bvh_nodes"] == len(nodes)
+    pierce.pj_free_dataset(ctx.h, h)
