@@ -55,3 +55,40 @@ def test_two_datasets(ctx):
     B = synth.urban(5005, n_buildings=3900, n_parts=400)
     c, k = _check(ctx, "urban x urban 4,300 x 4,300 meshes", A, B, False)
     assert c > 1000 and k > 100
+
+
+def _boxes(rng, n, side, span=(262143, 262143, 262143)):
+    lo = rng.integers(0, [max(1, s - d) for s, d in zip(span, side)], size=(n, 3))
+    hi = lo + rng.integers(1, np.array(side) + 1, size=(n, 3))
+    return [synth.box(tuple(a), tuple(np.minimum(b, 262143))) for a, b in zip(lo, hi)]
+
+
+@pytest.mark.parametrize("kind", ["sparse", "dense", "long", "huge", "two_sided", "one_bucket"])
+def test_sweep_over_box_shapes(ctx, kind):
+    # sparse: a few pairs a box; dense: more pairs than the list first has
+    # room for; long: ranges past the 16 steps of a box's own warp, thousands
+    # of them; huge: meshes with more pairs than are ordered in place;
+    # two_sided: few long boxes against many small ones; one_bucket: every
+    # low x in one bucket of 16 grid units
+    rng = np.random.default_rng(7)
+    B = None
+    if kind == "sparse":
+        A = _boxes(rng, 5900, (6000, 6000, 6000))
+    elif kind == "dense":
+        A = _boxes(rng, 5900, (30000, 60000, 60000))
+    elif kind == "long":
+        A = _boxes(rng, 5900, (200000, 2000, 2000))
+    elif kind == "huge":
+        A = [synth.box((k, 2 * k, 0), (262143 - k, 262143, 262143)) for k in range(1, 4)] + \
+            _boxes(rng, 5900, (3000, 3000, 3000))
+    elif kind == "two_sided":
+        A = _boxes(rng, 210, (90000, 5000, 5000))
+        B = _boxes(rng, 81000, (900, 900, 900))
+    else:
+        A = _boxes(rng, 5900, (9, 9000, 9000), (20, 262143, 262143))
+    A = synth.concat(A)
+    B = synth.concat(B) if B else None
+    c, k = _check(ctx, "sweep " + kind, A, B if B is not None else A, B is None)
+    assert c > 200 and k > 50
+    if kind == "dense":
+        assert c > 4 * 5900
