@@ -15,10 +15,10 @@
 // step sees the same candidate list.
 //
 // What bounds it: launches and one host wait (for the pairs' number, which
-// sizes the join's buffers); the sweep itself is about 40 us on 55,000 urban
+// sizes the join's buffers); the test pass is about 33 us on 55,000 urban
 // meshes.  Radix sorts of the boxes (4 passes) and of the pairs (8), the test
-// run twice and two host waits before this took 359 us there, 110 now
-// (267 and 80 on 6,007 x 9,001 cells and nuclei).  The sort of
+// run twice and two host waits before this took 359 us there, 116 now
+// (267 and 85 on 6,007 x 9,001 cells and nuclei).  The sort of
 // the pairs is still taken when a mesh has kSwMost pairs or more: ordering
 // its list compares all of them with each other.
 #include <cub/cub.cuh>
