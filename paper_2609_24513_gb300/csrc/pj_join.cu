@@ -1789,9 +1789,10 @@ __global__ void k_pred_combine(uint8_t *flags, const uint8_t *pflags, const int6
 // candidate pairs at once, so that every traversal round is wide: an expand
 // round copies the nodes of 16 (node, node) tasks (8 at W = 8) to shared
 // memory with asynchronous copies issued all at once and tests their child
-// pairs with 2 lanes per task (4 at W = 8); a leaf round does the same with
-// the triangles of up to 24 leaf pairs (48 / L), filters (edge, triangle)
-// tests by boxes and runs the exact tests that remain one per lane.  A round
+// pairs with 2 lanes per task (4 at W = 8); a leaf round reads the triangles
+// of 16 / L leaf pairs into registers, 2 L lanes to a pair, filters (edge,
+// triangle) tests by boxes and runs the exact tests that remain one per lane.
+// A round
 // thus waits for one memory latency however many fetches it makes.  A warp
 // takes new candidates whenever its stack holds less than one round.
 //
@@ -1852,22 +1853,12 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
 }
 
-// a staged triangle record (three float4, as in the BVH's triangle records)
-__device__ __forceinline__ void stage_tri(const float4 *stage, int i, F3 off, F3 &a, F3 &b,
-                                          F3 &c, int &own) {
-  const float4 r0 = stage[3 * i], r1 = stage[3 * i + 1], r2 = stage[3 * i + 2];
-  a = add(mkf3(r0.x, r0.y, r0.z), off);
-  b = add(mkf3(r0.w, r1.x, r1.y), off);
-  c = add(mkf3(r1.z, r1.w, r2.x), off);
-  own = __float_as_int(r2.y);
-}
-
-// Leaf rounds stage the triangles of up to kLeafPairs leaf pairs (at most
-// 48 / L) in shared memory: kStageF4 float4 = 4.5 KB per warp, which also
-// holds an expand round's nodes (16 or 8 tasks x 2 nodes x W slots, padded).
-constexpr int kLeafPairs = 24;
+// float4 of a warp's stage: an expand round's nodes (16 or 8 tasks x 2 nodes
+// x W slots, padded)
 constexpr int kStageF4 = 288;
-constexpr int kListMax = 384;  // queued (edge, triangle) tests: 32 units x 3 edges x 4 tests
+// listed (edge, triangle) tests of a warp, three words each: fewer than 32
+// are left over when a step of a leaf round adds up to 96
+constexpr int kListMax = 128;
 
 template <int W>
 struct StreamCfg {
@@ -1878,13 +1869,8 @@ struct StreamCfg {
   static_assert(NT * 2 * RS <= kStageF4, "an expand round's nodes must fit the stage");
   static constexpr int SC = W == 8 ? 384 : 192;                    // stack entries
   static constexpr int LQ = 64;                                    // leaf-pair entries
-  // per warp: stack, leaf queue (uint4 entries), triangle stage, boxes of
-  // the staged triangles and of the leaves, pair offsets, pair entries, hit
-  // words, test list
-  static constexpr int warp_bytes = (SC + LQ) * 16 + kStageF4 * 16 + kStageF4 / 3 * 6 * 4 +
-                                    kLeafPairs * 2 * 6 * 4 + kLeafPairs * 3 * 4 +
-                                    kLeafPairs * 16 + kLeafPairs * 4 + kLeafPairs * 4 +
-                                    kListMax * 2;
+  // per warp: stack, leaf queue (uint4 entries), node stage, test list
+  static constexpr int warp_bytes = (SC + LQ) * 16 + kStageF4 * 16 + kListMax * 12;
 };
 
 // control words of one launch (zeroed before it), each on its own 128-byte
@@ -1990,19 +1976,12 @@ __global__ void __launch_bounds__(128, 4) k_stream(StreamArgs P) {
   uint4 *stk = reinterpret_cast<uint4 *>(smem + (size_t)wib * Cf::warp_bytes);
   uint4 *lq = stk + Cf::SC;
   float4 *stage = reinterpret_cast<float4 *>(lq + Cf::LQ);
-  float *s_tbox = reinterpret_cast<float *>(stage + kStageF4);  // per staged triangle
-  float *s_box = s_tbox + kStageF4 / 3 * 6;                       // per leaf
-  float *s_off = s_box + kLeafPairs * 2 * 6;
-  uint4 *s_pe = reinterpret_cast<uint4 *>(s_off + kLeafPairs * 3);
-  volatile unsigned *s_hit = reinterpret_cast<volatile unsigned *>(s_pe + kLeafPairs);
-  float *s_err = reinterpret_cast<float *>(const_cast<unsigned *>(s_hit) + kLeafPairs);
-  unsigned short *s_list = reinterpret_cast<unsigned short *>(s_err + kLeafPairs);
+  unsigned *s_list = reinterpret_cast<unsigned *>(stage + kStageF4);
   const WaveArgs &Q = P.w;
   const unsigned lt = (1u << lane) - 1u;
   const int lsh = Q.lshift;
   const int L = 1 << lsh;                         // leaf size
-  const int pmax = min(kLeafPairs, 48 / L);       // leaf pairs per round (<= 32)
-  const int upi = L == 8 ? 16 : 32;               // leaf units per filter iteration
+  const int pmax = 16 / L;                        // leaf pairs per round: 2 L lanes each
   const F3 zero = mkf3(0.f, 0.f, 0.f);
   volatile const uint8_t *vflags = Q.flags;
   const int64_t n_in = *Q.n_cand;
@@ -2013,6 +1992,7 @@ __global__ void __launch_bounds__(128, 4) k_stream(StreamArgs P) {
   unsigned c_bx = 0;  // node bytes
   LeafCnt lc;
   int sp = 0, nlq = 0;
+  int ntest = 0;      // listed tests
   bool more = true;   // candidates may be left
   long long t_new = clock64();  // when this warp last took (or tried to take) work
   int err = DERR_NONE;
@@ -2082,216 +2062,132 @@ __global__ void __launch_bounds__(128, 4) k_stream(StreamArgs P) {
     }
   }
 
-  // one leaf round: the triangles of up to np leaf pairs from the top of the
-  // queue are copied to shared memory (cp.async, all at once), each leaf's
-  // box is taken from its triangles, every owned edge's box is tested against
-  // the other leaf's box and its triangles' boxes, and the surviving (edge,
-  // triangle) tests run one per lane.
+  // the last n (at most 32) listed tests, one per lane.  An entry is
+  // (candidate | bit 0 of the edge << 31, source triangle | side << 31,
+  // target triangle | bit 1 of the edge << 31); the records were read a moment
+  // ago by the round that listed it.
+  auto run_tests = [&](int n) {
+    ntest -= n;
+    if (lane < n) {
+      const unsigned *e = s_list + 3 * (ntest + lane);
+      const unsigned w0 = e[0], w1 = e[1], w2 = e[2];
+      const uint32_t c = w0 & 0x7FFFFFFFu;
+      const int k = (int)(w0 >> 31) | (int)(w2 >> 31 << 1);
+      const bool dir = w1 >> 31;
+      const F3 o = cand_offset(Q, c);
+      F3 v0, v1, v2, a, b, d;
+      int own, town;
+      load_tri(dir ? Q.B.trirec : Q.A.trirec, w1 & 0x7FFFFFFFu, dir ? o : zero, v0, v1, v2, own);
+      load_tri(dir ? Q.A.trirec : Q.B.trirec, w2 & 0x7FFFFFFFu, dir ? zero : o, a, b, d, town);
+      const F3 p = k == 0 ? v0 : (k == 1 ? v1 : v2);
+      const F3 q = k == 0 ? v1 : (k == 1 ? v2 : v0);
+      lc.st += 1;
+      bool r;
+      if (EXACT) {
+        r = segtri_exact_staged(p, q, a, b, d);
+      } else {
+        // the filter's bound from the box around the five points
+        const float dx = fmaxf(fmaxf(p.x, q.x), fmaxf(a.x, fmaxf(b.x, d.x))) -
+                         fminf(fminf(p.x, q.x), fminf(a.x, fminf(b.x, d.x)));
+        const float dy = fmaxf(fmaxf(p.y, q.y), fmaxf(a.y, fmaxf(b.y, d.y))) -
+                         fminf(fminf(p.y, q.y), fminf(a.y, fminf(b.y, d.y)));
+        const float dz = fmaxf(fmaxf(p.z, q.z), fmaxf(a.z, fmaxf(b.z, d.z))) -
+                         fminf(fminf(p.z, q.z), fminf(a.z, fminf(b.z, d.z)));
+        bool ex = false;
+        r = segtri_static(p, q, a, b, d, static_err(fmaxf(dx, fmaxf(dy, dz))), &ex);
+        lc.fb += ex ? 1 : 0;
+      }
+      if (r) Q.flags[c] = 1;
+    }
+    __syncwarp();
+  };
+
+  // One leaf round: up to pmax leaf pairs from the top of the queue, 2 L lanes
+  // to a pair, one source triangle (of either side) to a lane.  A lane reads
+  // its triangle and the other leaf's straight into registers, two targets at
+  // a time, and tests its owned edges' boxes against theirs; the surviving
+  // (edge, triangle) tests are listed and run 32 at a time, over rounds, so
+  // that the costly part has full warps.  Staging up to 24 pairs (48 / L) in
+  // shared memory for one round instead, their boxes computed there first and
+  // its tests run at its end, took 10,000-13,600 cycles a round and found a
+  // pair's crossing later: k_stream 238 -> 209 us on 10,000 x 500 tissue,
+  // 118 -> 87 on 2,311 x 117, 1,040 -> 945 on the instanced pairs (L = 4), 612
+  // -> 580 on the urban self join, 160 -> 145 on cells / nuclei.  (Five blocks
+  // per SM, which the smaller shared memory allows, spill at 96 registers:
+  // 250 us on the tissue.)
   auto leaf_round = [&]() {
     const int np = min(nlq, pmax);
-    uint4 pe = make_uint4(0u, 0u, 0u, 0u);
-    if (lane < np) {
-      pe = lq[nlq - 1 - lane];
-      s_pe[lane] = pe;
-    }
-    __syncwarp();
+    const int p = lane >> (lsh + 1), si = lane & (L - 1);
+    const bool dir = (lane >> lsh) & 1;
+    const bool in = p < np;
+    const uint4 e = in ? lq[nlq - 1 - p] : make_uint4(0u, 0u, 0u, 0u);
     nlq -= np;
-    // the pair's flag and offset load while the triangles are copied (a
-    // pair found intersecting meanwhile is copied for nothing)
-    uint8_t pfl = 1;
-    F3 po = zero;
-    if (lane < np) {
-      pfl = vflags[pe.x];
-      po = cand_offset(Q, pe.x);
-    }
-    // stage: the triangle records of each (pair p, side), contiguous in the
-    // mesh, go to float4 ((p * 2 + side) * L + t) * 3 + k.  A (pair, side)
-    // owns 4 L lanes of an iteration (at least its 3 L float4): lane h of
-    // them copies float4 h, so that the lanes of one run read consecutive
-    // addresses (one coalesced request per run instead of a lane copying it
-    // piece by piece).
-    {
-      const int chs = lsh + 2, h = lane & ((1 << chs) - 1);
-      for (int ps = lane >> chs; ps < 2 * np; ps += 32 >> chs) {
-        const int side = ps & 1;
-        const uint4 e = s_pe[ps >> 1];
-        const int n3 = 3 * ((int)((side ? e.w >> 8 : e.w) & 7u) + 1);
-        if (h < n3)
-          cp_async16(stage + 3 * (ps << lsh) + h,
-                     (side ? Q.B.trirec : Q.A.trirec) + 3 * (int64_t)(side ? e.z : e.y) + h);
-      }
-    }
-    if (lane < np) {
-      const bool alive = pfl == 0;
-      s_hit[lane] = alive ? 0u : 1u;
-      s_off[3 * lane] = po.x;
-      s_off[3 * lane + 1] = po.y;
-      s_off[3 * lane + 2] = po.z;
-      if (alive) {
-        lc.lp += 1;
-        lc.bytes += 48u * ((pe.w & 7u) + ((pe.w >> 8) & 7u) + 2u);
-      }
-    }
-    cp_async_wait_all();
-    __syncwarp();
-    // one lane per (pair, side): the boxes of the leaf's staged triangles
-    // (B's translated by the pair's offset) and the leaf's box; the two sides
-    // of a pair sit on adjacent lanes, which combine their leaf boxes into the
-    // pair's static filter bound (from the box around both leaves)
-    for (int ps0 = 0; ps0 < 2 * np; ps0 += 32) {
-      const int ps = ps0 + lane, p = ps >> 1, side = ps & 1;
-      float bx[6] = {3.4e38f, 3.4e38f, 3.4e38f, -3.4e38f, -3.4e38f, -3.4e38f};
-      const bool on = ps < 2 * np && !s_hit[p];  // the same for both sides
-      if (on) {
-        const uint4 e = s_pe[p];
-        const int n = (int)((side ? e.w >> 8 : e.w) & 7u) + 1;
-        const F3 o = side ? mkf3(s_off[3 * p], s_off[3 * p + 1], s_off[3 * p + 2]) : zero;
-        for (int t = 0; t < n; ++t) {
-          const int i = (ps << lsh) + t;
-          F3 a, b, c;
-          int own;
-          stage_tri(stage, i, o, a, b, c, own);
-          const float lx = fminf(a.x, fminf(b.x, c.x)), ly = fminf(a.y, fminf(b.y, c.y));
-          const float lz = fminf(a.z, fminf(b.z, c.z)), hx = fmaxf(a.x, fmaxf(b.x, c.x));
-          const float hy = fmaxf(a.y, fmaxf(b.y, c.y)), hz = fmaxf(a.z, fmaxf(b.z, c.z));
-          float *bp = s_tbox + 6 * i;
-          bp[0] = lx;
-          bp[1] = ly;
-          bp[2] = lz;
-          bp[3] = hx;
-          bp[4] = hy;
-          bp[5] = hz;
-          bx[0] = fminf(bx[0], lx);
-          bx[1] = fminf(bx[1], ly);
-          bx[2] = fminf(bx[2], lz);
-          bx[3] = fmaxf(bx[3], hx);
-          bx[4] = fmaxf(bx[4], hy);
-          bx[5] = fmaxf(bx[5], hz);
-        }
-        float *bp = s_box + 6 * ps;
+    const float4 *srec = dir ? Q.B.trirec : Q.A.trirec, *trec = dir ? Q.A.trirec : Q.B.trirec;
+    const uint32_t s0 = (dir ? e.z : e.y) + si, t0 = dir ? e.y : e.z;
+    const int ns = (int)((dir ? e.w >> 8 : e.w) & 7u) + 1;
+    int nt = (int)((dir ? e.w : e.w >> 8) & 7u) + 1;
+    const bool on = in && si < ns;
+    const uint8_t fl = on ? vflags[e.x] : (uint8_t)1;
+    const F3 po = on ? cand_offset(Q, e.x) : zero;
+    const F3 so = dir ? po : zero, to = dir ? zero : po;
+    F3 v[3] = {zero, zero, zero};
+    int own = 0;
+    if (on) load_tri(srec, s0, so, v[0], v[1], v[2], own);
+    F3 ta[2], tb[2], tc[2];
+    int town;
 #pragma unroll
-        for (int q = 0; q < 6; ++q) bp[q] = bx[q];
-      }
-      float ob[6];
-#pragma unroll
-      for (int q = 0; q < 6; ++q) ob[q] = __shfl_xor_sync(FULL, bx[q], 1);
-      if (on && side == 0) {
-        const float D = fmaxf(fmaxf(fmaxf(bx[3], ob[3]) - fminf(bx[0], ob[0]),
-                                    fmaxf(bx[4], ob[4]) - fminf(bx[1], ob[1])),
-                              fmaxf(bx[5], ob[5]) - fminf(bx[2], ob[2]));
-        s_err[p] = static_err(D);
-      }
+    for (int j = 0; j < 2; ++j)
+      if (on && j < nt) load_tri(trec, t0 + j, to, ta[j], tb[j], tc[j], town);
+    const bool alive = fl == 0;
+    if (!alive) own = 0;
+    if (alive && si == 0 && !dir) {
+      lc.lp += 1;
+      lc.bytes += 48u * (unsigned)(ns + nt);
     }
-    __syncwarp();
-    // the queued (edge, triangle) tests, one per lane: code = p | dir << 5 |
-    // s << 6 | k << 9 | t << 11
-    int nlist = 0;
-    auto flush = [&]() {
-      for (int i0 = 0; i0 < nlist; i0 += 32) {
-        const int i = i0 + lane;
-        if (i < nlist) {
-          const unsigned code = s_list[i];
-          const int p = code & 31, dir = (code >> 5) & 1, si = (code >> 6) & 7;
-          const int k = (code >> 9) & 3, t = (code >> 11) & 7;
-          // every shared-memory read of the test is issued at once, before
-          // the pair's hit word decides whether to run it
-          const F3 o = mkf3(s_off[3 * p], s_off[3 * p + 1], s_off[3 * p + 2]);
-          F3 v0, v1, v2, a, b, c;
-          int own, town;
-          stage_tri(stage, (p * 2 + dir) * L + si, dir ? o : zero, v0, v1, v2, own);
-          stage_tri(stage, (p * 2 + (dir ^ 1)) * L + t, dir ? zero : o, a, b, c, town);
-          const float err_p = s_err[p];
-          if (!s_hit[p]) {
-            const F3 pp = k == 0 ? v0 : (k == 1 ? v1 : v2);
-            const F3 qq = k == 0 ? v1 : (k == 1 ? v2 : v0);
-            lc.st += 1;
-            bool r;
-            if (EXACT) {
-              r = segtri_exact_staged(pp, qq, a, b, c);
-            } else {
-              bool ex = false;
-              r = segtri_static(pp, qq, a, b, c, err_p, &ex);
-              lc.fb += ex ? 1 : 0;
-            }
-            if (r) {
-              s_hit[p] = 1u;
-              Q.flags[s_pe[p].x] = 1;
-            }
+    lc.slab += (unsigned)__popc(own);
+    // boxes of the owned edges (open overlap is exact for crossings, see
+    // overlap_open; no slab test: its reciprocals cost more here than the
+    // exact tests it would save)
+    F3 elo[3], ehi[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const F3 a = v[k], b = v[k == 2 ? 0 : k + 1];
+      elo[k] = mkf3(fminf(a.x, b.x), fminf(a.y, b.y), fminf(a.z, b.z));
+      ehi[k] = mkf3(fmaxf(a.x, b.x), fmaxf(a.y, b.y), fmaxf(a.z, b.z));
+    }
+    for (int t = 0; t < L; t += 2) {
+      if (t > 0) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+          if (on && t + j < nt) load_tri(trec, t0 + t + j, to, ta[j], tb[j], tc[j], town);
+      }
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        if (t + j >= L) break;
+        const F3 lo = mkf3(fminf(ta[j].x, fminf(tb[j].x, tc[j].x)),
+                           fminf(ta[j].y, fminf(tb[j].y, tc[j].y)),
+                           fminf(ta[j].z, fminf(tb[j].z, tc[j].z)));
+        const F3 hi = mkf3(fmaxf(ta[j].x, fmaxf(tb[j].x, tc[j].x)),
+                           fmaxf(ta[j].y, fmaxf(tb[j].y, tc[j].y)),
+                           fmaxf(ta[j].z, fmaxf(tb[j].z, tc[j].z)));
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const bool keep = ((own >> k) & 1) && t + j < nt && lo.x < ehi[k].x &&
+                            elo[k].x < hi.x && lo.y < ehi[k].y && elo[k].y < hi.y &&
+                            lo.z < ehi[k].z && elo[k].z < hi.z;
+          const unsigned m = __ballot_sync(FULL, keep);
+          if (keep) {
+            unsigned *w = s_list + 3 * (ntest + __popc(m & lt));
+            w[0] = e.x | ((unsigned)(k & 1) << 31);
+            w[1] = s0 | ((unsigned)dir << 31);
+            w[2] = (t0 + t + j) | ((unsigned)(k >> 1) << 31);
           }
+          ntest += __popc(m);
         }
         __syncwarp();
+        while (ntest >= 32) run_tests(32);
       }
-      nlist = 0;
-    };
-    // units (p, dir, source triangle): the source's owned edges against the
-    // target leaf
-    const int nu = np * 2 * L;
-    for (int u0 = 0; u0 < nu; u0 += upi) {
-      const int u = lane < upi ? u0 + lane : nu;
-      unsigned mask = 0;  // bit k * L + t: edge k against target triangle t
-      int p = 0, dir = 0, si = 0;
-      if (u < nu) {
-        si = u & (L - 1);
-        const int pd = u >> lsh;
-        dir = pd & 1;
-        p = pd >> 1;
-        const uint4 e = s_pe[p];
-        const int ns = (int)((dir ? e.w >> 8 : e.w) & 7u) + 1;
-        const int nt = (int)((dir ? e.w : e.w >> 8) & 7u) + 1;
-        if (!s_hit[p] && si < ns) {
-          const F3 o = mkf3(s_off[3 * p], s_off[3 * p + 1], s_off[3 * p + 2]);
-          F3 v[3];
-          int own;
-          stage_tri(stage, (p * 2 + dir) * L + si, dir ? o : zero, v[0], v[1], v[2], own);
-          const float *bp = s_box + 6 * (p * 2 + (dir ^ 1));
-          const F3 tlo = mkf3(bp[0], bp[1], bp[2]), thi = mkf3(bp[3], bp[4], bp[5]);
-          const float *tbx = s_tbox + 6 * ((p * 2 + (dir ^ 1)) * L);
-          // box filters only (no slab test: its reciprocals cost more here
-          // than the exact tests it would save, which run one per lane)
-          // each owned edge's box against the leaf's (bit k of ek), then
-          // against each target triangle's box, read once for all edges
-          F3 elo[3], ehi[3];
-          unsigned ek = 0;
-#pragma unroll
-          for (int k = 0; k < 3; ++k) {
-            const F3 pp = v[k], qq = v[k == 2 ? 0 : k + 1];
-            elo[k] = mkf3(fminf(pp.x, qq.x), fminf(pp.y, qq.y), fminf(pp.z, qq.z));
-            ehi[k] = mkf3(fmaxf(pp.x, qq.x), fmaxf(pp.y, qq.y), fmaxf(pp.z, qq.z));
-            if (!((own >> k) & 1)) continue;
-            lc.slab += 1;
-            if (!(elo[k].x >= thi.x || tlo.x >= ehi[k].x || elo[k].y >= thi.y ||
-                  tlo.y >= ehi[k].y || elo[k].z >= thi.z || tlo.z >= ehi[k].z))
-              ek |= 1u << k;  // open overlap (exact for crossings, see overlap_open)
-          }
-          for (int t = 0; ek && t < nt; ++t) {
-            const float *tp = tbx + 6 * t;
-            const float t0 = tp[0], t1 = tp[1], t2 = tp[2], t3 = tp[3], t4 = tp[4], t5 = tp[5];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-              if (((ek >> k) & 1) && !(t0 >= ehi[k].x || elo[k].x >= t3 || t1 >= ehi[k].y ||
-                                       elo[k].y >= t4 || t2 >= ehi[k].z || elo[k].z >= t5))
-                mask |= 1u << (k * L + t);
-            }
-          }
-        }
-      }
-      // append this lane's tests (at most 3 L), flushing first if they would
-      // not fit
-      const int cnt = __popc(mask);
-      const int incl = warp_scan_incl(cnt, lane);
-      const int tot = __shfl_sync(FULL, incl, 31);
-      if (nlist + tot > kListMax) flush();
-      int pos = nlist + incl - cnt;
-      while (mask) {
-        const int b = __ffs(mask) - 1;
-        mask &= mask - 1;
-        const int k = b >> lsh, t = b & (L - 1);
-        s_list[pos++] = (unsigned short)(p | (dir << 5) | (si << 6) | (k << 9) | (t << 11));
-      }
-      nlist += tot;
-      __syncwarp();
     }
-    flush();
   };
 
   // take the k claimed queue entries at position h (their producers may
@@ -2416,6 +2312,7 @@ __global__ void __launch_bounds__(128, 4) k_stream(StreamArgs P) {
     }
     // 2. out of work: claim tasks from the queue, or leave
     if (sp == 0 && nlq == 0) {
+      if (ntest > 0) run_tests(ntest);
       if (more) continue;
       int64_t h = -1;
       int k = 0;
@@ -2482,7 +2379,7 @@ __global__ void __launch_bounds__(128, 4) k_stream(StreamArgs P) {
     // A full queue only ends the sharing: the warp keeps its work (all later
     // reservations fail too, so what is published stays a prefix).
     if (give && !q_full && sp >= Cf::NT / 2) q_full = !give_half(sp / 2);
-    if (give && !q_full && nlq >= pmax) q_full = !give_leaves(nlq / 2);
+    if (give && !q_full && nlq >= Cf::LQ / 2) q_full = !give_leaves(nlq / 2);
     // 4. leaf pairs once a round's worth is queued (or nothing else is left)
     if (nlq >= pmax || sp == 0) {
       leaf_round();
