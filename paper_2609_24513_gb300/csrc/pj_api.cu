@@ -42,9 +42,10 @@ pj_status cuda_fail(Ctx *c, cudaError_t e, const char *what) {
 }
 
 pj_status exec_init(Ctx *ctx, Exec *e) {
-  cudaError_t r = cudaMalloc(&e->d_err, sizeof(int) * 4);
-  if (r == cudaSuccess) r = cudaMemset(e->d_err, 0, sizeof(int) * 4);
-  if (r == cudaSuccess) r = cudaMallocHost(&e->h_pinned, 4096);
+  cudaError_t r = cudaMalloc(&e->d_misc, kExecBytes);
+  if (r == cudaSuccess) r = cudaMemset(e->d_misc, 0, kExecBytes);
+  if (r == cudaSuccess) e->d_err = reinterpret_cast<int *>(e->d_misc + 8);
+  if (r == cudaSuccess) r = cudaMallocHost(&e->h_pinned, 4096 + 8 * kFirstPairs);
   for (auto &ev : e->ev)
     if (r == cudaSuccess) r = cudaEventCreate(&ev);
   if (r != cudaSuccess) return cuda_fail(ctx, r, "exec_init");
@@ -60,10 +61,11 @@ void exec_free(Exec *e) {
     for (auto &kv : e->ws) cudaFree(kv.second.ptr);
   }
   e->ws.clear();
-  cudaFree(e->d_err);
+  cudaFree(e->d_misc);
   cudaFreeHost(e->h_pinned);
   for (auto &ev : e->ev)
     if (ev) cudaEventDestroy(ev);
+  e->d_misc = nullptr;
   e->d_err = nullptr;
   e->h_pinned = nullptr;
   for (auto &ev : e->ev) ev = nullptr;

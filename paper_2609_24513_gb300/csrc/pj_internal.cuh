@@ -104,8 +104,11 @@ struct Workspace {
 // API calls; each serving stream has its own.
 struct Exec {
   std::map<std::string, Workspace> ws;
-  int *d_err = nullptr;      // 4 device error words
-  void *h_pinned = nullptr;  // 4 KiB pinned host scratch
+  // kExecBytes of device memory: 8 words of a join's counts, then its 4 error
+  // words (cleared by one memset and read back by one copy)
+  int64_t *d_misc = nullptr;
+  int *d_err = nullptr;
+  void *h_pinned = nullptr;  // pinned host scratch: 4 KiB, then kFirstPairs pairs
   std::string err;           // last failure message of a serving thread
   bool borrow_out = false;   // join results stay in the workspaces (serving)
   cudaEvent_t ev[6] = {};    // a join's phase events, created once
@@ -113,6 +116,10 @@ struct Exec {
   // stream's order (null: the API calls' scratch, plain cudaMalloc)
   cudaStream_t stream = nullptr;
 };
+
+constexpr size_t kExecBytes = 128;
+// pairs of a host result that come back with the counts
+constexpr int64_t kFirstPairs = 32768;
 
 struct Serve;  // serving state (pj_serve.cu)
 
