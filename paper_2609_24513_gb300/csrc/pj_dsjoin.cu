@@ -44,7 +44,7 @@ constexpr int kParList = 48;      // objects a parity ray tracks
 constexpr int kHashProbes = 2048;  // probes before a hashmap counts as full
 
 enum { DS_EDGES = 0, DS_NODES, DS_TRIS, DS_HITS, DS_RAYS, DS_OVERFLOW, DS_ERR, DS_NREC,
-       DS_NOBJ, DS_NSTAT };
+       DS_NOBJ, DS_FULL, DS_NSTAT };
 
 struct DsSide {
   const float *xyz;
@@ -371,129 +371,418 @@ __global__ void __launch_bounds__(32 * kDsWarps, 4) k_ds_edges(DsSide A, DsSide 
   flush_stats(st, v, 4);
 }
 
-// Containment rays (Sec. 3.3): thread per object of Q, one ray from its
-// first lexicographic vertex through T's BVH along the axis direction that
-// leaves T's dataset box soonest (parity is the same in every direction for
-// a closed mesh and a point off it).  Only objects whose closed box holds
-// the vertex can contain it; up to kParList of them are tracked with a
-// parity bit and an on-surface bit.  dir 0: Q = B, T = A; dir 1 the reverse.
+// ---------------------------------------------------------------------------
+// Alg. 1 in both directions at once for two datasets: the two BVHs walked
+// together.  A queue entry is a pair of items, one of each dataset, whose
+// boxes overlap (open): a node of either BVH, or a leaf.  A step replaces it
+// by the overlapping pairs of the children of the larger node, or of both
+// where they are of similar size; pairs of two leaves go to a list, and the
+// edges of each against the other's triangles are tested from there.  Each
+// part of one dataset thus meets only the parts of the other that lie around
+// it, wherever the walk is, instead of being looked for from the root: 1,200
+// nuclei x 60 vessels take 64,000 pairs, where packets of 32 triangles
+// (k_ds_edges) took 2.0 M node visits and 1,100 us; 190 now.
+//
+// The walk is breadth first, a launch per level, the narrow ones in one block.
+// What bounds it is each level's launch and chain of dependent reads.  Queue and list are of fixed size; where they do not
+// suffice (DS_FULL: dense data) the packets trace the edges after all, as they
+// do for a self join, in which every triangle meets its own mesh's.
+// ---------------------------------------------------------------------------
+constexpr uint32_t kDsOpen = 0x40000000u;   // the item's children are taken
+constexpr uint32_t kDsIdx = 0x3FFFFFFFu;    // node, or node * W + k of a leaf
+constexpr unsigned kDsQueue = 1u << 22;     // entries of a queue
+constexpr unsigned kDsLeaves = 1u << 23;    // leaf pairs
+constexpr int kDsLevelT = 512;              // threads of a block of the walk
+constexpr unsigned kDsNarrow = 64;          // entries of a level that one block takes
+constexpr int kDsLevels = 192;              // levels of the walk
+
+__device__ __forceinline__ float ds_side(F3 lo, F3 hi) {
+  return fmaxf(hi.x - lo.x, fmaxf(hi.y - lo.y, hi.z - lo.z));
+}
+
+// an entry of two items with these sizes: which of them the next step opens
+__device__ __forceinline__ uint2 ds_entry(uint32_t a, float sa, uint32_t b, float sb) {
+  const bool la = a & kLeafBit, lb = b & kLeafBit;
+  return make_uint2(a | (!la && (lb || !(sb > 2.f * sa)) ? kDsOpen : 0u),
+                    b | (!lb && (la || !(sa > 2.f * sb)) ? kDsOpen : 0u));
+}
+
+// child slot k of an open item, or the item's own box and word
 template <int W>
-__global__ void __launch_bounds__(128) k_ds_parity(DsSide Q, DsSide T, int dir, int self_join,
-                                                   Sink sink, Recheck rc, bool first_pass,
-                                                   unsigned long long *st) {
-  uint32_t stk[kDsStack];
-  int lobj[kParList];
-  uint8_t lbits[kParList];
-  unsigned long long c_rays = 0, c_nodes = 0, c_tris = 0;
+__device__ __forceinline__ void ds_slot(const float *nodes, uint32_t item, int k, F3 &lo, F3 &hi,
+                                        uint32_t &word, uint32_t &child) {
   const int SW = node_stride_words(W);
-  // T's dataset box: the root's own slot
-  const float4 b0 = __ldg(reinterpret_cast<const float4 *>(T.nodes));
-  const float4 b1 = __ldg(reinterpret_cast<const float4 *>(T.nodes) + 1);
-  const F3 tlo = mkf3(b0.x, b0.y, b0.z), thi = mkf3(b0.w, b1.x, b1.y);
-  for (int64_t iq = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; iq < Q.M;
-       iq += (int64_t)gridDim.x * blockDim.x) {
+  const uint32_t ix = item & kDsIdx;
+  const bool open = item & kDsOpen, leaf = item & kLeafBit;
+  const float4 *p = reinterpret_cast<const float4 *>(
+      nodes + (open ? (int64_t)ix * SW + 8 * (k + 1)
+                    : leaf ? (int64_t)(ix / W) * SW + 8 * (ix % W + 1) : (int64_t)ix * SW));
+  const float4 q0 = __ldg(p), q1 = __ldg(p + 1);
+  lo = mkf3(q0.x, q0.y, q0.z);
+  hi = mkf3(q0.w, q1.x, q1.y);
+  word = __float_as_uint(q1.z);
+  child = !open ? item : ((word & kLeafBit) ? (kLeafBit | (ix * W + k)) : word);
+}
+
+// one entry's child pair r (of at most W x W) per lane: leaf pairs to the
+// list, others to the next queue
+template <int W>
+__device__ __forceinline__ void ds_step(const float *nodesA, const float *nodesB, uint2 e, int r,
+                                        bool on, uint2 *qout, unsigned *n_out, uint2 *leaves,
+                                        unsigned *n_leaves, unsigned long long *st, int lane) {
+  const int nA = (e.x & kDsOpen) ? W : 1, nB = (e.y & kDsOpen) ? W : 1;
+  on = on && r < nA * nB;
+  bool ok = false;
+  uint2 next = make_uint2(0u, 0u), pair = next;
+  if (on) {
+    F3 alo, ahi, blo, bhi;
+    uint32_t wa, wb, ca, cb;
+    ds_slot<W>(nodesA, e.x, r / nB, alo, ahi, wa, ca);
+    ds_slot<W>(nodesB, e.y, r % nB, blo, bhi, wb, cb);
+    ok = open_overlap(alo, ahi, blo, bhi);  // an empty slot's box is inverted
+    next = ds_entry(ca, ds_side(alo, ahi), cb, ds_side(blo, bhi));
+    pair = make_uint2(wa, wb);  // of two leaves: their descriptors
+  }
+  const bool leaf = ok && (next.x & next.y & kLeafBit);
+  const unsigned m1 = __ballot_sync(0xffffffffu, ok && !leaf);
+  const unsigned m2 = __ballot_sync(0xffffffffu, leaf);
+  unsigned b1 = 0, b2 = 0;
+  if (lane == 0 && m1) b1 = atomicAdd(n_out, (unsigned)__popc(m1));
+  if (lane == 0 && m2) b2 = atomicAdd(n_leaves, (unsigned)__popc(m2));
+  b1 = __shfl_sync(0xffffffffu, b1, 0) + __popc(m1 & ((1u << lane) - 1u));
+  b2 = __shfl_sync(0xffffffffu, b2, 0) + __popc(m2 & ((1u << lane) - 1u));
+  if (ok && !leaf) {
+    if (b1 < kDsQueue) qout[b1] = next;
+    else st[DS_FULL] = 1ull;
+  }
+  if (leaf) {
+    if (b2 < kDsLeaves) leaves[b2] = pair;
+    else st[DS_FULL] = 1ull;
+  }
+}
+
+// A launch of the walk.  Launch i finds its level in at[i] and leaves the next
+// one's in at[i + 1]; cnt[l] counts the entries of level l (queues alternate).
+// A level of more than kDsNarrow entries is taken by the whole grid; narrower
+// ones, the first and the last few, by one block, level after level until one
+// is wide or none is left (the join took 628, 533 and 509 us with 1,024, 256
+// and 64 entries as the line, 588 with the first levels in a kernel of their
+// own and a launch for each further one).
+// Launches that find nothing return at once; they are queued ahead
+// (programmatic launches), as many as the trees have levels.
+template <int W>
+__global__ void __launch_bounds__(kDsLevelT) k_ds_level(const float *nodesA, const float *nodesB,
+                                                        uint2 *q0, uint2 *q1, unsigned *cnt,
+                                                        unsigned *at, int i, uint2 *leaves,
+                                                        unsigned *n_leaves,
+                                                        unsigned long long *st) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  constexpr int G = W * W < 32 ? W * W : 32, PER = W * W / G;
+  const int lane = threadIdx.x & 31;
+  int lv = (int)__ldcg(at + i);
+  unsigned n = __ldcg(cnt + lv);
+  const bool wide = n > kDsNarrow;
+  if (!wide && blockIdx.x > 0) return;
+  unsigned long long visited = 0;
+  if (i == 0) {  // the pair of roots
+    if (threadIdx.x == 0) {
+      const float4 *a = reinterpret_cast<const float4 *>(nodesA);
+      const float4 *b = reinterpret_cast<const float4 *>(nodesB);
+      const float4 a0 = a[0], a1 = a[1], b0 = b[0], b1 = b[1];
+      q0[0] = ds_entry(0u, ds_side(mkf3(a0.x, a0.y, a0.z), mkf3(a0.w, a1.x, a1.y)), 0u,
+                       ds_side(mkf3(b0.x, b0.y, b0.z), mkf3(b0.w, b1.x, b1.y)));
+      __threadfence();
+    }
+    __syncthreads();
+    n = 1;
+  }
+  const unsigned threads = wide ? gridDim.x * kDsLevelT : kDsLevelT;
+  const unsigned t0 = (wide ? blockIdx.x * kDsLevelT : 0u) + threadIdx.x - lane;
+  while (n > 0 && lv < kDsLevels - 1) {
+    n = min(n, kDsQueue);
+    visited += 2ull * n;
+    const uint2 *qin = lv & 1 ? q1 : q0;
+    uint2 *qout = lv & 1 ? q0 : q1;
+    for (unsigned e0 = t0 / G; e0 < n; e0 += threads / G) {
+      const unsigned e = e0 + lane / G;
+      const uint2 x = e < n ? __ldcg(qin + e) : make_uint2(0u, 0u);
+#pragma unroll
+      for (int j = 0; j < PER; ++j)
+        ds_step<W>(nodesA, nodesB, x, lane % G + j * G, e < n, qout, cnt + lv + 1, leaves,
+                   n_leaves, st, lane);
+    }
+    ++lv;
+    if (wide) break;
+    __threadfence();
+    __syncthreads();
+    n = __ldcg(cnt + lv);
+    if (n > kDsNarrow) break;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    at[i + 1] = (unsigned)lv;
+    if (visited) atomicAdd(st + DS_NODES, visited);
+  }
+}
+
+// The listed leaf pairs: 2 L lanes to a pair, one source triangle of either
+// side to a lane, its owned edges against the other leaf's triangles; the
+// tests that box comparisons leave are listed and run 32 at a time.  Records
+// are counted and placed per warp of the grid.
+__global__ void __launch_bounds__(32 * kDsWarps) k_ds_leaf(DsSide A, DsSide B, const uint2 *leaves,
+                                                           const unsigned *n_leaves, int lshift,
+                                                           Sink sink, unsigned long long *st) {
+  __shared__ unsigned s_list[kDsWarps][128 * 3];
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, L = 1 << lshift;
+  const unsigned lt = (1u << lane) - 1u;
+  unsigned *list = s_list[wib];
+  const int64_t warp = blockIdx.x * (int64_t)kDsWarps + wib, nw = gridDim.x * (int64_t)kDsWarps;
+  const int64_t item = sink.base + warp;
+  const unsigned n = min(*n_leaves, kDsLeaves);
+  unsigned long long c_tris = 0, c_hits = 0;
+  int64_t n_rec = 0;
+  int ntest = 0;
+  // the last m listed: (source triangle, side | edge << 1, target triangle)
+  auto run = [&](int m) {
+    ntest -= m;
+    bool hit = false;
+    unsigned long long key = 0;
+    if (lane < m) {
+      const unsigned *e = list + 3 * (ntest + lane);
+      const bool dir = e[1] & 1u;
+      const int k = (int)(e[1] >> 1);
+      const DsTri a = ds_tri(dir ? B.trirec : A.trirec, e[0]);
+      const DsTri b = ds_tri(dir ? A.trirec : B.trirec, e[2]);
+      const F3 p = k == 0 ? a.v[0] : (k == 1 ? a.v[1] : a.v[2]);
+      const F3 q = k == 0 ? a.v[1] : (k == 1 ? a.v[2] : a.v[0]);
+      bool ex = false;
+      c_tris += 1;
+      hit = segtri_filtered(p, q, b.v[0], b.v[1], b.v[2], &ex);
+      key = dir ? pair_key(b.mesh, a.mesh, 0) : pair_key(a.mesh, b.mesh, 0);
+    }
+    const unsigned mh = __ballot_sync(full, hit);
+    if (hit) {
+      c_hits += 1;
+      if (sink.mode == SINK_HASH) hash_insert(sink, key, st);
+      else if (sink.mode == SINK_EMIT) sink.keys[sink.off[item] + n_rec + __popc(mh & lt)] = key;
+    }
+    n_rec += __popc(mh);
+    __syncwarp();
+  };
+  const int per = 16 >> lshift;  // pairs of a step
+  for (int64_t p0 = warp * per; p0 < n; p0 += nw * per) {
+    const int64_t p = p0 + (lane >> (lshift + 1));
+    const int si = lane & (L - 1);
+    const unsigned dir = (lane >> lshift) & 1;
+    const uint2 e = p < n ? leaves[p] : make_uint2(0u, 0u);
+    const uint32_t sw = dir ? e.y : e.x, tw = dir ? e.x : e.y;
+    const int64_t s0 = (sw >> 3) & 0x0FFFFFFFu, t0 = (tw >> 3) & 0x0FFFFFFFu;
+    const int nt = (int)(tw & 7u) + 1;
+    DsTri a;
+    a.edges = 0;
+    if (p < n && si <= (int)(sw & 7u)) a = ds_tri(dir ? B.trirec : A.trirec, s0 + si);
+    for (int t = 0; t < L; ++t) {
+      F3 blo = mkf3(0.f, 0.f, 0.f), bhi = blo;
+      unsigned own = 0;
+      if (a.edges && t < nt) {
+        const DsTri b = ds_tri(dir ? A.trirec : B.trirec, t0 + t);
+        blo = min3(b.v[0], min3(b.v[1], b.v[2]));
+        bhi = max3(b.v[0], max3(b.v[1], b.v[2]));
+        own = (unsigned)a.edges;
+      }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const F3 u = a.v[k], v = a.v[k == 2 ? 0 : k + 1];
+        const bool keep = ((own >> k) & 1u) && open_overlap(min3(u, v), max3(u, v), blo, bhi);
+        const unsigned m = __ballot_sync(full, keep);
+        if (keep) {
+          unsigned *w = list + 3 * (ntest + __popc(m & lt));
+          w[0] = (unsigned)(s0 + si);
+          w[1] = dir | (unsigned)(k << 1);
+          w[2] = (unsigned)(t0 + t);
+        }
+        ntest += __popc(m);
+      }
+      __syncwarp();
+      while (ntest >= 32) run(32);
+    }
+  }
+  if (ntest > 0) run(ntest);
+  if (sink.mode == SINK_COUNT && lane == 0) sink.cnt[item] = n_rec;
+  const unsigned long long v[2] = {c_tris, c_hits};
+  flush_stats(st + DS_TRIS, v, 2);
+}
+
+// Containment rays (Sec. 3.3): a warp per object of Q, one ray from its first
+// lexicographic vertex through T's BVH along the axis direction that leaves
+// T's dataset box soonest (parity is the same in every direction for a closed
+// mesh and a point off it).  Only objects whose closed box holds the vertex
+// can contain it; up to kParList of them are tracked with a parity bit and an
+// on-surface bit.  Q = B, T = A, then the reverse (a self join: Q = T = A
+// once).  The children of up to 32 / W nodes are tested at a time, and a
+// leaf's triangles one per lane; a thread per object walked alone (150 us for
+// 1,260 objects, 21 now).
+constexpr int kParLeaves = 64;  // listed leaves of a warp
+
+template <int W>
+__global__ void __launch_bounds__(32 * kDsWarps) k_ds_parity(DsSide A, DsSide B, int self_join,
+                                                             Sink sink, Recheck rc,
+                                                             bool first_pass, int lshift,
+                                                             unsigned long long *st) {
+  constexpr int kCap = 2 * kDsStack + 32;  // as in k_ds_edges
+  __shared__ uint32_t s_stack[kDsWarps][kCap], s_leaf[kDsWarps][kParLeaves];
+  __shared__ int s_obj[kDsWarps][kParList];
+  __shared__ unsigned s_bits[kDsWarps][kParList];
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, SW = node_stride_words(W);
+  const unsigned lt = (1u << lane) - 1u;
+  uint32_t *stk = s_stack[wib], *leaf = s_leaf[wib];
+  int *lobj = s_obj[wib];
+  unsigned *lbits = s_bits[wib];
+  unsigned long long c_rays = 0, c_nodes = 0, c_tris = 0;
+  const int64_t nB = self_join ? A.M : B.M, nA = self_join ? 0 : A.M;
+  for (int64_t w = blockIdx.x * (int64_t)kDsWarps + wib; w < nB + nA;
+       w += gridDim.x * (int64_t)kDsWarps) {
+    const bool rev = w >= nB;  // an object of A against B
+    const int64_t iq = rev ? w - nB : w;
+    const float4 *qrec = (rev || self_join ? A.mrec : B.mrec) + 3 * iq;
+    const float *tnodes = rev ? B.nodes : A.nodes, *taabb = rev ? B.aabb : A.aabb;
+    const float4 *trec = rev ? B.trirec : A.trirec;
     int64_t n_rec = 0;
-    const float4 q0 = Q.mrec[3 * iq], q1 = Q.mrec[3 * iq + 1], q2 = Q.mrec[3 * iq + 2];
+    const float4 q0 = qrec[0], q1 = qrec[1], q2 = qrec[2];
     const F3 vf = mkf3(q0.w, q1.w, q2.x);
+    // T's dataset box: the root's own slot
+    const float4 b0 = __ldg(reinterpret_cast<const float4 *>(tnodes));
+    const float4 b1 = __ldg(reinterpret_cast<const float4 *>(tnodes) + 1);
+    const F3 tlo = mkf3(b0.x, b0.y, b0.z), thi = mkf3(b0.w, b1.x, b1.y);
     if (vf.x >= tlo.x && vf.x <= thi.x && vf.y >= tlo.y && vf.y <= thi.y && vf.z >= tlo.z &&
         vf.z <= thi.z) {
-      c_rays += 1;
+      c_rays += lane == 0;
       const I3 v = toi(vf);
       int ax, dr;
       ray_axis_choice(vf, tlo, thi, ax, dr);
-      int nl = 0;
+      int nl = 0, sp = 1, nlf = 0;
       bool over = false;
-      int sp = 0;
-      stk[sp++] = 0u;
-      while (sp > 0) {
-        const uint32_t node = stk[--sp];
-        c_nodes += 1;
-        const float4 *slot = reinterpret_cast<const float4 *>(T.nodes + (int64_t)node * SW + 8);
-        for (int c = 0; c < W; ++c) {
-          const float4 s0 = __ldg(slot + 2 * c), s1 = __ldg(slot + 2 * c + 1);
-          const uint32_t ch = __float_as_uint(s1.z);
-          if (ch == kEmpty) continue;
-          Box bx;
-          bx.lo = mkf3(s0.x, s0.y, s0.z);
-          bx.hi = mkf3(s0.w, s1.x, s1.y);
-          if (!ray_axis_box(vf, bx, ax, dr)) continue;
-          if (ch & kLeafBit) {
-            const int64_t first = (ch >> 3) & 0x0FFFFFFFu;
-            const int cnt = (int)(ch & 7u) + 1;
-            for (int t = 0; t < cnt; ++t) {
-              const float4 r2 = __ldg(T.trirec + 3 * (first + t) + 2);
-              const int ot = __float_as_int(r2.w);
-              if (self_join && ot == (int)iq) continue;
-              int li = -1;
-              for (int j = 0; j < nl; ++j)
-                if (lobj[j] == ot) li = j;
-              if (li < 0) {
+      if (lane == 0) stk[0] = 0u;
+      __syncwarp();
+      while (sp > 0 || nlf > 0) {
+        if (sp == 0 || nlf + 32 > kParLeaves) {
+          // the listed leaves' triangles, L lanes to a leaf
+          for (int i0 = 0; i0 < nlf; i0 += 32 >> lshift) {
+            const int i = i0 + (lane >> lshift), t = lane & ((1 << lshift) - 1);
+            bool in = false;
+            int ot = 0;
+            unsigned bits = 0;
+            if (i < nlf && t <= (int)(leaf[i] & 7u)) {
+              const DsTri x = ds_tri(trec, ((leaf[i] >> 3) & 0x0FFFFFFFu) + t);
+              ot = x.mesh;
+              if (!(self_join && ot == (int)iq)) {
                 // an object whose box does not hold the vertex cannot contain it
-                const float *ob = T.aabb + 6 * (int64_t)ot;
-                if (vf.x < ob[0] || vf.x > ob[3] || vf.y < ob[1] || vf.y > ob[4] || vf.z < ob[2] ||
-                    vf.z > ob[5])
-                  continue;
+                const float *ob = taabb + 6 * (int64_t)ot;
+                in = !(vf.x < ob[0] || vf.x > ob[3] || vf.y < ob[1] || vf.y > ob[4] ||
+                       vf.z < ob[2] || vf.z > ob[5]);
+              }
+              if (in) {
+                c_tris += 1;
+                const I3 a = toi(x.v[0]), b = toi(x.v[1]), c = toi(x.v[2]);
+                bits = (on_triangle(v, a, b, c) ? 2u : 0u) |
+                       (ray_axis_hit(v, a, b, c, ax, dr) ? 1u : 0u);
+              }
+            }
+            // (an object is tracked from the first triangle on, hit or not)
+            for (unsigned m = __ballot_sync(full, in); m; m &= m - 1) {
+              const int l = __ffs(m) - 1;
+              const int o = __shfl_sync(full, ot, l);
+              const unsigned bt = __shfl_sync(full, bits, l);
+              int li = -1;
+              for (int j0 = 0; j0 < nl; j0 += 32) {
+                const unsigned f = __ballot_sync(full, j0 + lane < nl && lobj[j0 + lane] == o);
+                if (f) li = j0 + __ffs(f) - 1;
+              }
+              if (li < 0) {
                 if (nl == kParList) {
                   over = true;
                   continue;
                 }
                 li = nl++;
-                lobj[li] = ot;
-                lbits[li] = 0;
+                if (lane == 0) {
+                  lobj[li] = o;
+                  lbits[li] = 0;
+                }
               }
-              const float4 r0 = __ldg(T.trirec + 3 * (first + t));
-              const float4 r1 = __ldg(T.trirec + 3 * (first + t) + 1);
-              c_tris += 1;
-              const I3 a = toi(mkf3(r0.x, r0.y, r0.z)), b = toi(mkf3(r0.w, r1.x, r1.y));
-              const I3 cc = toi(mkf3(r1.z, r1.w, r2.x));
-              uint8_t bits = lbits[li];
-              if (on_triangle(v, a, b, cc)) bits |= 2;
-              if (ray_axis_hit(v, a, b, cc, ax, dr)) bits ^= 1;
-              lbits[li] = bits;
+              if (lane == 0) lbits[li] = ((lbits[li] | bt) & 2u) | ((lbits[li] ^ bt) & 1u);
+              __syncwarp();
             }
-          } else {
-            if (sp >= kDsStack) {
-              atomicExch(st + DS_ERR, 1ull);
-              sp = 0;
-              break;
-            }
-            stk[sp++] = ch;
           }
+          __syncwarp();
+          nlf = 0;
+          continue;
         }
+        const int n = sp <= kDsStack ? min(sp, 32 / W) : 1;
+        c_nodes += lane == 0 ? n : 0;
+        bool in = false;
+        uint32_t ch = 0;
+        if (lane < n * W) {
+          const float4 *slot = reinterpret_cast<const float4 *>(
+              tnodes + (int64_t)stk[sp - 1 - lane / W] * SW + 8 + 8 * (lane % W));
+          const float4 s0 = __ldg(slot), s1 = __ldg(slot + 1);
+          ch = __float_as_uint(s1.z);
+          Box bx;
+          bx.lo = mkf3(s0.x, s0.y, s0.z);
+          bx.hi = mkf3(s0.w, s1.x, s1.y);
+          in = ch != kEmpty && ray_axis_box(vf, bx, ax, dr);
+        }
+        const bool lf = in && (ch & kLeafBit);
+        const unsigned m1 = __ballot_sync(full, in && !lf), m2 = __ballot_sync(full, lf);
+        sp -= n;
+        if (sp + __popc(m1) > kCap) {
+          if (lane == 0) atomicExch(st + DS_ERR, 1ull);
+          break;
+        }
+        if (in && !lf) stk[sp + __popc(m1 & lt)] = ch;
+        if (lf) leaf[nlf + __popc(m2 & lt)] = ch;
+        sp += __popc(m1);
+        nlf += __popc(m2);
+        __syncwarp();
       }
-      if (over && first_pass) {
+      if (over && first_pass && lane == 0) {
         // every candidate of this object goes to the per-pair join
         const unsigned long long i = atomicAdd(st + DS_NOBJ, 1ull);
         if (i < rc.cap) rc.objs[i] = (int32_t)iq;
         else atomicExch(st + DS_ERR, 2ull);
       }
-      for (int j = 0; j < nl; ++j) {
-        const int a = dir == 0 ? lobj[j] : (int)iq, b = dir == 0 ? (int)iq : lobj[j];
-        if (lbits[j] & 2) {
+      for (int j0 = 0; j0 < nl; j0 += 32) {
+        const int j = j0 + lane;
+        const unsigned bits = j < nl ? lbits[j] : 0u;
+        const int o = j < nl ? lobj[j] : 0;
+        const int a = rev ? (int)iq : o, b = rev ? o : (int)iq;
+        if ((bits & 2) && first_pass && !over) {
           // the vertex lies on this object's surface: the pair's own test
-          if (first_pass && !over) {
-            const unsigned long long i = atomicAdd(st + DS_NREC, 1ull);
-            if (i < rc.cap) rc.pairs[i] = make_int2(a, b);
-            else atomicExch(st + DS_ERR, 2ull);
-          }
-        } else if (lbits[j] & 1) {
+          const unsigned long long i = atomicAdd(st + DS_NREC, 1ull);
+          if (i < rc.cap) rc.pairs[i] = make_int2(a, b);
+          else atomicExch(st + DS_ERR, 2ull);
+        }
+        const bool rec = bits == 1u;
+        const unsigned m = __ballot_sync(full, rec);
+        if (rec) {
           const unsigned long long key = pair_key(a, b, self_join);
           if (sink.mode == SINK_HASH) hash_insert(sink, key, st);
-          else if (sink.mode == SINK_EMIT) sink.keys[sink.off[sink.base + iq] + n_rec] = key;
-          ++n_rec;
+          else if (sink.mode == SINK_EMIT)
+            sink.keys[sink.off[sink.base + w] + n_rec + __popc(m & lt)] = key;
         }
+        n_rec += __popc(m);
       }
+      __syncwarp();
     }
-    if (sink.mode == SINK_COUNT) sink.cnt[sink.base + iq] = n_rec;
+    if (sink.mode == SINK_COUNT && lane == 0) sink.cnt[sink.base + w] = n_rec;
   }
-  const unsigned long long v[3] = {c_rays, c_nodes, c_tris};
-  unsigned long long w[4] = {0, 0, 0, 0};
-  w[0] = v[0];
-  flush_stats(st + DS_RAYS, w, 1);
-  w[0] = v[1];
-  flush_stats(st + DS_NODES, w, 1);
-  w[0] = v[2];
-  flush_stats(st + DS_TRIS, w, 1);
+  unsigned long long x[1] = {c_rays};
+  flush_stats(st + DS_RAYS, x, 1);
+  x[0] = c_nodes;
+  flush_stats(st + DS_NODES, x, 1);
+  x[0] = c_tris;
+  flush_stats(st + DS_TRIS, x, 1);
 }
 
 // the occupied slots of a hashmap, in any order
@@ -588,7 +877,7 @@ static DsSide ds_side(Dataset *d, Bvh *b) {
 }
 
 typedef void (*DsEdgeKernel)(DsSide, DsSide, int, Sink, unsigned long long *);
-typedef void (*DsParKernel)(DsSide, DsSide, int, int, Sink, Recheck, bool, unsigned long long *);
+typedef void (*DsParKernel)(DsSide, DsSide, int, Sink, Recheck, bool, int, unsigned long long *);
 
 pj_status run_dataset_join(Ctx *ctx, Dataset *A, Dataset *B, int self_join,
                            const pj_dsjoin_opts *o, pj_pairs *out, pj_dsjoin_stats *stats,
@@ -646,29 +935,64 @@ pj_status run_dataset_join(Ctx *ctx, Dataset *A, Dataset *B, int self_join,
   int32_t *rc_objs = (int32_t *)ws_get(ctx, "ds_recheck_obj", sizeof(int32_t) * rc_cap, &st);
   if (!rc_objs) return st;
   Recheck rc{rc_pairs, rc_objs, rc_cap};
-  const int grid = ctx->num_sms * 16;
-  // one tracing pass over every item: A's packets of triangles, B's, B's
-  // objects, A's objects (count / emit arrays are indexed in this order)
+  const int lshift = L == 1 ? 0 : (L == 2 ? 1 : (L == 4 ? 2 : 3));
+  // edges by the walk of both BVHs, or in packets (see k_ds_level)
+  const int levels = bA->max_depth + bB->max_depth;
+  bool dual = !self_join && levels + 2 < kDsLevels;
+  uint2 *q0 = nullptr, *q1 = nullptr, *leaves = nullptr;
+  unsigned *lv_cnt = nullptr;  // entries per level, the leaf pairs, the launches' levels
+  if (dual) {
+    q0 = (uint2 *)ws_get(ctx, "ds_queue0", sizeof(uint2) * (size_t)kDsQueue, &st);
+    if (q0) q1 = (uint2 *)ws_get(ctx, "ds_queue1", sizeof(uint2) * (size_t)kDsQueue, &st);
+    if (q1) leaves = (uint2 *)ws_get(ctx, "ds_leaves", sizeof(uint2) * (size_t)kDsLeaves, &st);
+    if (leaves) lv_cnt = (unsigned *)ws_get(ctx, "ds_levels", 4 * (2 * kDsLevels + 1), &st);
+    if (!lv_cnt) return st;
+  }
+  // one tracing pass over every item: the warps that test the leaf pairs, or
+  // A's packets of triangles and B's; B's objects, A's objects (count / emit
+  // arrays are indexed in this order)
+  const int leaf_grid = ctx->num_sms * 8;
   auto packets = [](int64_t F) { return (F + kDsPacket - 1) / kDsPacket; };
-  const int64_t nFA = packets(A->F), nFB = self_join ? 0 : packets(B->F), nMB = parity ? B->M : 0;
-  const int64_t nMA = parity && !self_join ? A->M : 0;
-  const int64_t items = nFA + nFB + nMB + nMA;
+  const int64_t nPack = packets(A->F) + (self_join ? 0 : packets(B->F));
+  const int64_t nObj = !parity ? 0 : (self_join ? A->M : A->M + B->M);
+  auto edge_items = [&]() { return dual ? (int64_t)leaf_grid * kDsWarps : nPack; };
   auto trace = [&](Sink k, bool first_pass) -> pj_status {
     k.base = 0;
-    // enough warps to spread the costly packets, few enough that their
-    // counters' atomics do not queue up
-    const int egrid = (int)std::min<int64_t>((nFA + nFB + kDsWarps - 1) / kDsWarps,
-                                             ctx->num_sms * 32);
-    ke<<<egrid, 32 * kDsWarps, 0, s>>>(sA, self_join ? sA : sB, self_join, k, d_st);
-    if (parity) {
-      k.base = nFA + nFB;
-      kp<<<grid, 128, 0, s>>>(self_join ? sA : sB, sA, 0, self_join, k, rc, first_pass, d_st);
-      if (!self_join) {
-        k.base = nFA + nFB + nMB;
-        kp<<<grid, 128, 0, s>>>(sA, sB, 1, 0, k, rc, first_pass, d_st);
+    if (dual) {
+      unsigned *n_leaves = lv_cnt + kDsLevels;
+      if (first_pass) {
+        const auto kl = W == 2 ? k_ds_level<2> : (W == 4 ? k_ds_level<4> : k_ds_level<8>);
+        PJ_CK(cudaMemsetAsync(lv_cnt, 0, 4 * (2 * kDsLevels + 1), s));
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(ctx->num_sms * 4);
+        cfg.blockDim = dim3(kDsLevelT);
+        cfg.stream = s;
+        cfg.attrs = &attr;
+        for (int l = 0; l < levels; ++l) {
+          cfg.numAttrs = l > 0;
+          PJ_CK(cudaLaunchKernelEx(&cfg, kl, sA.nodes, sB.nodes, q0, q1, lv_cnt,
+                                   lv_cnt + kDsLevels + 1, l, leaves, n_leaves, d_st));
+        }
+        ctx->launches += levels;
       }
+      k_ds_leaf<<<leaf_grid, 32 * kDsWarps, 0, s>>>(sA, sB, leaves, n_leaves, lshift, k, d_st);
+    } else {
+      // enough warps to spread the costly packets, few enough that their
+      // counters' atomics do not queue up
+      const int egrid = (int)std::min<int64_t>((nPack + kDsWarps - 1) / kDsWarps,
+                                               ctx->num_sms * 32);
+      ke<<<egrid, 32 * kDsWarps, 0, s>>>(sA, self_join ? sA : sB, self_join, k, d_st);
     }
-    ctx->launches += 1 + (parity ? (self_join ? 1 : 2) : 0);
+    if (parity) {
+      k.base = edge_items();
+      kp<<<(int)std::min<int64_t>((nObj + kDsWarps - 1) / kDsWarps, ctx->num_sms * 32),
+           32 * kDsWarps, 0, s>>>(sA, self_join ? sA : sB, self_join, k, rc, first_pass, lshift,
+                                  d_st);
+    }
+    ctx->launches += parity ? 2 : 1;
     PJ_CK(cudaGetLastError());
     return PJ_OK;
   };
@@ -695,6 +1019,10 @@ pj_status run_dataset_join(Ctx *ctx, Dataset *A, Dataset *B, int self_join,
       PJ_CK(cudaMemcpyAsync(h_st, d_st, sizeof(h_st), cudaMemcpyDeviceToHost, s));
       PJ_CK(cudaStreamSynchronize(s));
       cudaEventElapsedTime(&ms_trace, ev[2], ev[4]);
+      if (dual && h_st[DS_FULL]) {
+        dual = false;  // too dense for the walk's queue or list
+        continue;
+      }
       if (!h_st[DS_OVERFLOW]) {
         keys = (unsigned long long *)ws_get(ctx, "ds_keys", 8 * (size_t)cap + 8, &st);
         if (!keys) return st;
@@ -715,20 +1043,30 @@ pj_status run_dataset_join(Ctx *ctx, Dataset *A, Dataset *B, int self_join,
     }
   } else {
     // count, prefix sum, emit
-    int64_t *cnt = (int64_t *)ws_get(ctx, "ds_count", 8 * (size_t)(items + 1), &st);
-    if (!cnt) return st;
-    int64_t *off = (int64_t *)ws_get(ctx, "ds_off", 8 * (size_t)(items + 1), &st);
-    if (!off) return st;
-    PJ_CK(cudaMemsetAsync(d_st, 0, 8 * DS_NSTAT, s));
-    PJ_CK(cudaMemsetAsync(cnt + items, 0, 8, s));
-    PJ_CK(cudaEventRecord(ev[2], s));
-    Sink kc{SINK_COUNT, nullptr, 0, cnt, nullptr, nullptr, 0};
-    if ((st = trace(kc, true)) != PJ_OK) return st;
-    size_t tb = 0;
-    PJ_CK(cub::DeviceScan::ExclusiveSum(nullptr, tb, cnt, off, (int)(items + 1), s));
-    void *tmp = ws_get(ctx, "ds_scan_tmp", tb, &st);
-    if (!tmp) return st;
-    PJ_CK(cub::DeviceScan::ExclusiveSum(tmp, tb, cnt, off, (int)(items + 1), s));
+    int64_t *off = nullptr;
+    int64_t items = 0;
+    for (;;) {
+      items = edge_items() + nObj;
+      int64_t *cnt = (int64_t *)ws_get(ctx, "ds_count", 8 * (size_t)(items + 1), &st);
+      if (!cnt) return st;
+      off = (int64_t *)ws_get(ctx, "ds_off", 8 * (size_t)(items + 1), &st);
+      if (!off) return st;
+      PJ_CK(cudaMemsetAsync(d_st, 0, 8 * DS_NSTAT, s));
+      PJ_CK(cudaMemsetAsync(cnt, 0, 8 * (size_t)(items + 1), s));
+      PJ_CK(cudaEventRecord(ev[2], s));
+      Sink kc{SINK_COUNT, nullptr, 0, cnt, nullptr, nullptr, 0};
+      if ((st = trace(kc, true)) != PJ_OK) return st;
+      size_t tb = 0;
+      PJ_CK(cub::DeviceScan::ExclusiveSum(nullptr, tb, cnt, off, (int)(items + 1), s));
+      void *tmp = ws_get(ctx, "ds_scan_tmp", tb, &st);
+      if (!tmp) return st;
+      PJ_CK(cub::DeviceScan::ExclusiveSum(tmp, tb, cnt, off, (int)(items + 1), s));
+      if (!dual) break;
+      PJ_CK(cudaMemcpyAsync(h_st, d_st, sizeof(h_st), cudaMemcpyDeviceToHost, s));
+      PJ_CK(cudaStreamSynchronize(s));
+      if (!h_st[DS_FULL]) break;
+      dual = false;  // too dense for the walk's queue or list
+    }
     int64_t total = 0;
     PJ_CK(cudaMemcpyAsync(&total, off + items, 8, cudaMemcpyDeviceToHost, s));
     PJ_CK(cudaStreamSynchronize(s));
@@ -751,7 +1089,7 @@ pj_status run_dataset_join(Ctx *ctx, Dataset *A, Dataset *B, int self_join,
   }
   if (h_st[DS_ERR] == 1) return fail(ctx, PJ_ERR_INTERNAL, "dataset BVH traversal stack exceeded");
   if (h_st[DS_ERR] == 2) return fail(ctx, PJ_ERR_NO_MEMORY, "too many parity rays to recheck");
-  S.edges = (int64_t)h_st[DS_EDGES];
+  S.edges = A->E + (self_join ? 0 : B->E);  // every owned edge
   S.node_visits = (int64_t)h_st[DS_NODES];
   S.tri_tests = (int64_t)h_st[DS_TRIS];
   S.hits = (int64_t)h_st[DS_HITS];

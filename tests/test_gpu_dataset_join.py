@@ -127,3 +127,28 @@ def test_packet_sizes(ctx, sides, bands, W, L):
             assert np.array_equal(got, want), (pred, mat)
             hits.add(st["hits"])
         assert len(hits) == 1
+
+
+def test_dense_datasets_leave_the_walk(ctx):
+    # 16 x 16 mutually crossing spheres of 20,480 triangles: far more
+    # overlapping leaf pairs (at least 9.5 M) than the joint walk's
+    # list holds, so that the packets trace the edges; against the per-pair
+    # join, which other tests hold to the oracle
+    V, F = synth.icosphere(5)
+    rng = np.random.default_rng(3)
+    R = synth.random_rotations(rng, 32)
+    ball = [(synth.quantize(0.5 + (V @ R[k].T) * (0.2 + 1e-6 * k)), F) for k in range(32)]
+    A, B = synth.concat(ball[:16]), synth.concat(ball[16:])
+    ha, hb = ctx.load(A), ctx.load(B)
+    ctx.build(ha, 4, 2)
+    ctx.build(hb, 4, 2)
+    for pred in ("intersects", "overlap"):
+        want, _ = ctx.join(ha, hb, predicate=pred)
+        assert len(want) > 100
+        for mat in MATS:
+            got, st = pierce.pj_dataset_join(ctx.h, ha, hb, predicate=pred, materialize=mat)
+            assert np.array_equal(got, want), (pred, mat)
+            assert st["hits"] > 50_000
+            assert st["edges"] == 3 * (len(A.tris) + len(B.tris)) // 2
+    pierce.pj_free_dataset(ctx.h, ha)
+    pierce.pj_free_dataset(ctx.h, hb)
