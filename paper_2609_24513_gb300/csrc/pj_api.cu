@@ -578,6 +578,32 @@ void free_dataset(Ctx *ctx, Dataset *d) {
     mem_put(ctx, p, ctx->stream);
 }
 
+pj_status mesh_boxes(Ctx *ctx, const float *xyz, const int64_t *voff, int64_t M, float *box,
+                     bool *ok) {
+  cudaStream_t s = ctx->stream;
+  const int64_t v0 = voff[0], V = voff[M] - v0;
+  std::vector<int64_t> off(voff, voff + M + 1);
+  for (auto &o : off) o -= v0;
+  TmpMem tmp(ctx, s);
+  int64_t *d_off;
+  float *d_box;
+  unsigned long long *d_bad, bad = 0;
+  PJ_CK(tmp.get(&d_off, M + 1));
+  PJ_CK(tmp.get(&d_box, 6 * M));
+  PJ_CK(tmp.get(&d_bad, 1));
+  PJ_CK(cudaMemcpyAsync(d_off, off.data(), sizeof(int64_t) * (M + 1), cudaMemcpyHostToDevice, s));
+  PJ_CK(cudaMemsetAsync(d_bad, 0xff, 8, s));
+  k_init_aabb<<<nblk(ctx, 6 * M), 256, 0, s>>>(d_box, M);
+  k_validate_boxes<<<span_blocks(V), 256, 0, s>>>(xyz + 3 * v0, V, d_off, M,
+                                                  reinterpret_cast<int *>(d_box), d_bad);
+  PJ_CK(cudaGetLastError());
+  PJ_CK(cudaMemcpyAsync(box, d_box, sizeof(float) * 6 * M, cudaMemcpyDeviceToHost, s));
+  PJ_CK(cudaMemcpyAsync(&bad, d_bad, 8, cudaMemcpyDeviceToHost, s));
+  PJ_CK(cudaStreamSynchronize(s));
+  *ok = bad == ~0ull;
+  return PJ_OK;
+}
+
 pj_status load_impl(Ctx *ctx, const float *xyz, int64_t V,
                            const int32_t *tris, int64_t F, const int64_t *voff,
                            const int64_t *toff, int64_t M, int dev_ptrs,

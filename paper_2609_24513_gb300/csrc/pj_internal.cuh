@@ -240,6 +240,11 @@ enum { DERR_NONE = 0, DERR_STACK = 1, DERR_QUEUE = 2, DERR_OFFSET = 3, DERR_TIME
 
 // build.cu
 pj_status build_bvh(Ctx *ctx, Dataset *ds, int W, int L, cudaStream_t s);
+// closed boxes of M meshes (host) whose coordinates xyz the device can read,
+// mesh k's vertices being [voff[k], voff[k + 1]); *ok: every coordinate is an
+// integer on the grid (else the boxes are not to be used)
+pj_status mesh_boxes(Ctx *ctx, const float *xyz, const int64_t *voff, int64_t M, float *box,
+                     bool *ok);
 // (the device must be done with the BVH / dataset)
 void free_bvh(Ctx *ctx, Bvh &b);
 // tune.cu

@@ -65,3 +65,18 @@ def test_pathology_full_under_a_budget(ctx, pathology_truth):
           "%.0f ms (device %.0f, gather %.0f overlapped)"
           % (st["grid"], st["cells_joined"], st["mesh_copies"], st["max_cell_bytes"] / 1e9,
              st["ms_total"], st["ms_device"], st["ms_gather"]))
+
+
+def test_meshes_that_start_inside_their_arrays(ctx):
+    # offsets need not start at 0, nor coordinates be on the grid for a mesh
+    # that no cell loads; one that is loaded is refused as ever
+    A, B = synth.tiny_spheres(1003)
+    want = oracle.join_all(A, B)
+    cut = synth.MeshSet(A.xyz, A.tris, A.voff[3:], A.toff[3:])
+    got, _ = pierce.pj_join_tiled(ctx.h, cut, B, grid=3)
+    assert np.array_equal(got, want[want[:, 0] >= 3] - [3, 0])
+    bad = synth.MeshSet(A.xyz.copy(), A.tris, A.voff, A.toff)
+    bad.xyz[5, 1] += 0.5
+    with pytest.raises(pierce.PierceError) as e:
+        pierce.pj_join_tiled(ctx.h, bad, B, grid=2)
+    assert e.value.code == 2                          # PJ_ERR_NOT_QUANTIZED
