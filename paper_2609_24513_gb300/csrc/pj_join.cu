@@ -1813,14 +1813,16 @@ __global__ void k_pred_combine(uint8_t *flags, const uint8_t *pflags, const int6
 // tasks from the queue; a straggler -- a warp that has not been able to take
 // new work for `give_after` SM cycles, while most warps take some every few
 // rounds -- that sees more than `hungry_min` hungry warps (a few that wait
-// cost less than the tasks' way through the queue: with any, 1,120 / 800 us
-// on the instanced pairs and the urban join against 1,040 / 612) gives the
+// cost less than the tasks' way through the queue: with any, with a quarter,
+// a half and three quarters of a warp per SM the urban join took 800, 727,
+// 570 and 541 us, the instanced pairs 1,120, 1,105, 945 and 926) gives the
 // older half of its stack (the larger subtrees) to the queue, and so does a
 // warp whose stack is nearly full.  A costly pair thus spreads over more and more warps.  At most
 // `hungry_max` warps wait for tasks (a warp that finds that many waiting
 // leaves): a heavy pair needs tens of helpers, not thousands of warps
-// polling the same words (a cap of 4 per SM; with 2 per SM 4,429 x 260
-// tissue within at W = 8 took 270 us, with 4 252, the others the same).  A crossing sets the candidate's flag; the tasks
+// polling the same words (a cap of 6 per SM; with 2 per SM 4,429 x 260
+// tissue within at W = 8 took 270 us, with 4 252; 200 x 200 spheres took 200
+// us with 4, 181 with 6; the others the same).  A crossing sets the candidate's flag; the tasks
 // of a flagged candidate are dropped when popped or claimed.
 //
 // Queue protocol.  Entries are uint4 (candidate, item A, item B, ready).  A
@@ -3012,8 +3014,8 @@ static PairParityKernel pick_pair_parity(int W);  // defined with its kernel
 
 // when the streaming launch's warps share work (measured beside the kernel)
 static void stream_limits(const Ctx *ctx, StreamArgs &sa) {
-  sa.hungry_max = 4u * (unsigned)ctx->num_sms;
-  sa.hungry_min = (unsigned)ctx->num_sms / 2;
+  sa.hungry_max = 6u * (unsigned)ctx->num_sms;
+  sa.hungry_min = 3u * (unsigned)ctx->num_sms / 4u;
   sa.give_after = 2000;
 }
 
