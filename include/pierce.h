@@ -379,7 +379,8 @@ typedef struct {
                                kept in the one cell that holds its reference
                                point                                          */
   float ms_total;           /* wall time of the whole join                   */
-  float ms_gather;          /* host time gathering cells (overlapped)        */
+  float ms_gather;          /* host time gathering cells (overlapped; 0 where
+                               the device gathers them itself)                */
   float ms_device;          /* load, BVH build and join of the cells         */
   float reserved2;
 } pj_tiled_stats;
@@ -387,10 +388,12 @@ typedef struct {
 /* A join of two datasets that need not fit in device memory: a coarse grid
  * over both datasets' box, each mesh copied to every cell its closed box
  * touches, the cells loaded, indexed and joined one after another with the
- * same kernels as pj_join_intersects_ex (the next cell is gathered on the
- * host while the current one runs).  A pair is kept only in the cell that
- * holds the lower corner of its two boxes' intersection, a point of both
- * boxes, so every pair is reported exactly once.  Global mesh ids, sorted.
+ * same kernels as pj_join_intersects_ex.  Where the device can read pageable
+ * host memory through the host's page tables it gathers each cell's meshes
+ * from the caller's arrays itself; elsewhere the host gathers the next cell
+ * while the current one runs.  A pair is kept only in the cell that holds the
+ * lower corner of its two boxes' intersection, a point of both boxes, so
+ * every pair is reported exactly once.  Global mesh ids, sorted.
  * self_join: b is ignored (a with itself, pairs i < j).  A mesh larger than
  * the budget fails with PJ_ERR_NO_MEMORY.  Synchronous. */
 pj_status pj_join_tiled(pj_ctx *ctx, const pj_host_meshes *a, const pj_host_meshes *b,
@@ -423,7 +426,9 @@ typedef struct {
 
 typedef struct {
   int64_t edges;            /* owned edges traced (both directions)          */
-  int64_t node_visits;      /* BVH nodes visited by edges and parity rays    */
+  int64_t node_visits;      /* BVH nodes read: two per node pair of the joint
+                               walk, one per node an edge packet or a parity
+                               ray visits                                     */
   int64_t tri_tests;        /* strict segment/triangle tests                 */
   int64_t hits;             /* crossings found, repeats included             */
   int64_t parity_rays;      /* one per object with a vertex in the other box */
@@ -442,11 +447,13 @@ typedef struct {
 
 /* The join as the paper formulates it, without candidate pairs: one BVH
  * over all triangles of each dataset (built and cached per W, L on first
- * use); every owned edge of A traced as a bounded segment through B's BVH
- * and every owned edge of B through A's (Alg. 1 both ways, Sec. 3.2), every
- * strict crossing recorded (the multi-hit loop: an edge may pierce several
- * objects) as the pair (idA, idB), duplicates merged by the chosen
- * materialisation (Sec. 3.5).  For PJ_PRED_INTERSECTS each object also casts
+ * use); every owned edge of A tested as a bounded segment against B's
+ * triangles and every owned edge of B against A's (Alg. 1 both ways, Sec.
+ * 3.2) by walking the two BVHs together (a self join, or data too dense for
+ * the walk's queue, sends the edges through the BVH in packets of 32
+ * triangles), every strict crossing recorded (the multi-hit loop: an edge may
+ * pierce several objects) as the pair (idA, idB), duplicates merged by the
+ * chosen materialisation (Sec. 3.5).  For PJ_PRED_INTERSECTS each object also casts
  * one parity ray from its lexicographically first vertex against the other
  * dataset's BVH, toggling a parity bit per object it crosses (Sec. 3.3-3.4);
  * odd parity with the vertex off that object's surface records the pair.
