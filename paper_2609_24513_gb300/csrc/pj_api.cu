@@ -701,10 +701,10 @@ pj_status load_impl(Ctx *ctx, const float *xyz, int64_t V,
     uint2 *list;
     PJ_CK(tmp.get(&list, 3 * F));
     size_t tb = 0;
-    PJ_CK(cub::DeviceScan::ExclusiveSum(nullptr, tb, deg, deg_off, (int)(V + 1), s));
+    PJ_CK(cub::DeviceScan::ExclusiveSum(nullptr, tb, deg, deg_off, V + 1, s));
     char *tstore;
     PJ_CK(tmp.get(&tstore, (int64_t)tb));
-    PJ_CK(cub::DeviceScan::ExclusiveSum(tstore, tb, deg, deg_off, (int)(V + 1), s));
+    PJ_CK(cub::DeviceScan::ExclusiveSum(tstore, tb, deg, deg_off, V + 1, s));
     PJ_CK(cudaMemsetAsync(d->d_emask, 0, (size_t)(F + 3) / 4 * 4, s));
     k_edge_lists<<<nblk(ctx, F), 256, 0, s>>>(d->d_tris, F, deg_off, rank, list);
     if (V > 0)

@@ -946,7 +946,7 @@ pj_status run_dataset_join(Ctx *ctx, Dataset *A, Dataset *B, int self_join,
     if (q0) q1 = (uint2 *)ws_get(ctx, "ds_queue1", sizeof(uint2) * (size_t)kDsQueue, &st);
     if (q1) leaves = (uint2 *)ws_get(ctx, "ds_leaves", sizeof(uint2) * (size_t)kDsLeaves, &st);
     if (leaves) lv_cnt = (unsigned *)ws_get(ctx, "ds_levels", 4 * (2 * kDsLevels + 1), &st);
-    if (!lv_cnt) return st;
+    if (!lv_cnt) dual = false;  // no room for the walk's 136 MB: the packets need none
   }
   // one tracing pass over every item: the warps that test the leaf pairs, or
   // A's packets of triangles and B's; B's objects, A's objects (count / emit
