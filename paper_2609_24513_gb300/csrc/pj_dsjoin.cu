@@ -424,12 +424,42 @@ __device__ __forceinline__ void ds_slot(const float *nodes, uint32_t item, int k
   child = !open ? item : ((word & kLeafBit) ? (kLeafBit | (ix * W + k)) : word);
 }
 
+// A warp's part of a list: entries wait in shared memory until there are 32
+// for one reservation.  A reservation per step, of about two entries, queued
+// the wide levels up at the list's counter: 10,000 nuclei x 500 vessels, 3.9 M
+// entries, took 2.07 ms of walk, leaves and rays; 1.34 now, the widest level
+// 352 us and now 129 (1,200 x 60: the join 485 and now 471).
+struct DsOut {
+  uint2 *buf;  // 64 entries
+  int n;       // of them waiting
+  uint2 *list;
+  unsigned *count, cap;
+  __device__ __forceinline__ void put(bool on, unsigned m, uint2 e, unsigned long long *st,
+                                      int lane) {
+    if (on) buf[n + __popc(m & ((1u << lane) - 1u))] = e;
+    n += __popc(m);
+    if (n >= 32) flush(32, st, lane);
+  }
+  __device__ __forceinline__ void flush(int k, unsigned long long *st, int lane) {
+    __syncwarp();
+    unsigned at = 0;
+    if (lane == 0) at = atomicAdd(count, (unsigned)k);
+    at = __shfl_sync(0xffffffffu, at, 0) + lane;
+    n -= k;
+    if (lane < k) {
+      if (at < cap) list[at] = buf[n + lane];
+      else st[DS_FULL] = 1ull;
+    }
+    __syncwarp();
+  }
+};
+
 // one entry's child pair r (of at most W x W) per lane: leaf pairs to the
 // list, others to the next queue
 template <int W>
 __device__ __forceinline__ void ds_step(const float *nodesA, const float *nodesB, uint2 e, int r,
-                                        bool on, uint2 *qout, unsigned *n_out, uint2 *leaves,
-                                        unsigned *n_leaves, unsigned long long *st, int lane) {
+                                        bool on, DsOut &next_q, DsOut &leaf_q,
+                                        unsigned long long *st, int lane) {
   const int nA = (e.x & kDsOpen) ? W : 1, nB = (e.y & kDsOpen) ? W : 1;
   on = on && r < nA * nB;
   bool ok = false;
@@ -446,19 +476,8 @@ __device__ __forceinline__ void ds_step(const float *nodesA, const float *nodesB
   const bool leaf = ok && (next.x & next.y & kLeafBit);
   const unsigned m1 = __ballot_sync(0xffffffffu, ok && !leaf);
   const unsigned m2 = __ballot_sync(0xffffffffu, leaf);
-  unsigned b1 = 0, b2 = 0;
-  if (lane == 0 && m1) b1 = atomicAdd(n_out, (unsigned)__popc(m1));
-  if (lane == 0 && m2) b2 = atomicAdd(n_leaves, (unsigned)__popc(m2));
-  b1 = __shfl_sync(0xffffffffu, b1, 0) + __popc(m1 & ((1u << lane) - 1u));
-  b2 = __shfl_sync(0xffffffffu, b2, 0) + __popc(m2 & ((1u << lane) - 1u));
-  if (ok && !leaf) {
-    if (b1 < kDsQueue) qout[b1] = next;
-    else st[DS_FULL] = 1ull;
-  }
-  if (leaf) {
-    if (b2 < kDsLeaves) leaves[b2] = pair;
-    else st[DS_FULL] = 1ull;
-  }
+  if (m1) next_q.put(ok && !leaf, m1, next, st, lane);
+  if (m2) leaf_q.put(leaf, m2, pair, st, lane);
 }
 
 // A launch of the walk.  Launch i finds its level in at[i] and leaves the next
@@ -479,7 +498,10 @@ __global__ void __launch_bounds__(kDsLevelT) k_ds_level(const float *nodesA, con
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   constexpr int G = W * W < 32 ? W * W : 32, PER = W * W / G;
+  __shared__ uint2 s_buf[kDsLevelT / 32][2][64];
   const int lane = threadIdx.x & 31;
+  uint2 *buf = s_buf[threadIdx.x >> 5][0];
+  DsOut leaf_q{buf + 64, 0, leaves, n_leaves, kDsLeaves};
   int lv = (int)__ldcg(at + i);
   unsigned n = __ldcg(cnt + lv);
   const bool wide = n > kDsNarrow;
@@ -503,15 +525,15 @@ __global__ void __launch_bounds__(kDsLevelT) k_ds_level(const float *nodesA, con
     n = min(n, kDsQueue);
     visited += 2ull * n;
     const uint2 *qin = lv & 1 ? q1 : q0;
-    uint2 *qout = lv & 1 ? q0 : q1;
+    DsOut next_q{buf, 0, lv & 1 ? q0 : q1, cnt + lv + 1, kDsQueue};
     for (unsigned e0 = t0 / G; e0 < n; e0 += threads / G) {
       const unsigned e = e0 + lane / G;
       const uint2 x = e < n ? __ldcg(qin + e) : make_uint2(0u, 0u);
 #pragma unroll
       for (int j = 0; j < PER; ++j)
-        ds_step<W>(nodesA, nodesB, x, lane % G + j * G, e < n, qout, cnt + lv + 1, leaves,
-                   n_leaves, st, lane);
+        ds_step<W>(nodesA, nodesB, x, lane % G + j * G, e < n, next_q, leaf_q, st, lane);
     }
+    if (next_q.n > 0) next_q.flush(next_q.n, st, lane);
     ++lv;
     if (wide) break;
     __threadfence();
@@ -519,6 +541,7 @@ __global__ void __launch_bounds__(kDsLevelT) k_ds_level(const float *nodesA, con
     n = __ldcg(cnt + lv);
     if (n > kDsNarrow) break;
   }
+  if (leaf_q.n > 0) leaf_q.flush(leaf_q.n, st, lane);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     at[i + 1] = (unsigned)lv;
     if (visited) atomicAdd(st + DS_NODES, visited);
