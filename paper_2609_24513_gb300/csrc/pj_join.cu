@@ -3650,7 +3650,10 @@ pj_status run_join(Ctx *ctx, Dataset *A, Dataset *B, const int32_t *cand,
            (int)o->launch_mode, (long long)Ccap, (int)budget1,
            args.max_pop * 1000 + wave_levels * 2 + (stream ? 1 : 0),
            (mbb_in_graph ? 1 + self_join : 0) + 4 * pred);
-  snprintf(gk + strlen(gk), sizeof(gk) - strlen(gk), "|%d", (int)o->wait_polls);
+  // whether the sequence clears the flags itself: a sweep's list and a host
+  // list of the same length share every buffer and count
+  snprintf(gk + strlen(gk), sizeof(gk) - strlen(gk), "|%d|%d", (int)o->wait_polls,
+           (int)flags_clear);
   bool replayed = false;
   if (graph) {
     auto it = ctx->graphs.find(gk);

@@ -92,3 +92,29 @@ def test_sweep_over_box_shapes(ctx, kind):
     assert c > 200 and k > 50
     if kind == "dense":
         assert c > 4 * 5900
+
+
+def test_sweep_graph_beside_a_host_list_graph(ctx):
+    # a sweep join and a join over a host list of the same length use the same
+    # buffers, but only the latter's flags are cleared before its graph runs:
+    # the sweep must not replay the list's graph over another join's flags
+    U = synth.urban(5003, n_buildings=5600, n_parts=600)
+    h = ctx.load(U)
+    ctx.build(h, 4, 2)
+    want, info = ctx.join(h, h, self_join=True)
+    n = info["n_candidates"]
+    cand = oracle.mbb_candidates(U, U, self_join=True)
+    assert n == len(cand) and 100 < len(want) < n
+    flags = oracle_flags("sweep beside a list", U, U, cand).astype(bool)
+    assert np.array_equal(want, cand[flags])
+    order = np.random.default_rng(11).permutation(n)
+    for _ in range(2):                                    # captured, then replayed
+        got, _ = ctx.join(h, h, cand=cand[order], use_graph=True)
+        assert np.array_equal(got, cand[order][flags[order]])
+    # every flag set by an unrelated join of the same length
+    ctx.join(h, h, cand=want[np.arange(n) % len(want)])
+    for _ in range(2):
+        got, _ = ctx.join(h, h, self_join=True, use_graph=True)
+        assert np.array_equal(got, want)
+    got, _ = ctx.join(h, h, cand=cand[order], use_graph=True)
+    assert np.array_equal(got, cand[order][flags[order]])
