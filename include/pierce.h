@@ -637,6 +637,21 @@ pj_status pj_export_bvh(pj_ctx *ctx, pj_dataset ds, int32_t width,
 pj_status pj_export_mesh_data(pj_ctx *ctx, pj_dataset ds, float *aabb,
                               int32_t *lex_first, uint8_t *edge_owner);
 
+/* For tests: limits that let small data reach paths taken only on large data,
+ * after a failure or on another machine.  Zero-initialised = none. */
+typedef struct {
+  int32_t noalloc_polls;    /* pj_join_intersects_noalloc: bound on the polls of
+                               each wait of the streaming kernel (as
+                               pj_join_opts.wait_polls)                      */
+  int32_t noalloc_queue;    /* and entries of its task queue that it uses    */
+  int32_t tiled_host_gather; /* 1: pj_join_tiled works out boxes and gathers
+                               cells on the host even where the device can    */
+  int32_t reserved;
+} pj_test_limits;
+
+/* Set a context's test limits (NULL: none). */
+pj_status pj_set_test_limits(pj_ctx *ctx, const pj_test_limits *limits);
+
 #ifdef __cplusplus
 }
 #endif

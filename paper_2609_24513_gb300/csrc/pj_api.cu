@@ -1137,6 +1137,14 @@ pj_status pj_autotune(pj_ctx *h, pj_dataset a, pj_dataset b, const int32_t *cand
   return st;
 }
 
+pj_status pj_set_test_limits(pj_ctx *h, const pj_test_limits *limits) {
+  Ctx *ctx = reinterpret_cast<Ctx *>(h);
+  if (!ctx) return PJ_ERR_INVALID_ARG;
+  std::lock_guard<std::mutex> lk(ctx->mu);
+  ctx->limits = limits ? *limits : pj_test_limits{};
+  return PJ_OK;
+}
+
 pj_status pj_get_counters(pj_ctx *h, pj_counters *out) {
   Ctx *ctx = reinterpret_cast<Ctx *>(h);
   if (!ctx || !out) return PJ_ERR_INVALID_ARG;

@@ -135,6 +135,7 @@ struct Ctx {
   unsigned long long *d_counters = nullptr;  // C_NUM
   Exec main;                                 // scratch of the API calls
   pj_config cfg{};
+  pj_test_limits limits{};                   // zero outside tests
   // captured graphs keyed by a shape string, with their kernel counts
   std::map<std::string, cudaGraphExec_t> graphs;
   std::map<std::string, unsigned long long> graph_kernels;

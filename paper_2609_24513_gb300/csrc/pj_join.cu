@@ -4074,7 +4074,9 @@ pj_status run_join_noalloc(Ctx *ctx, Dataset *A, Dataset *B, const int32_t *d_ca
     sa.ctl = reinterpret_cast<unsigned int *>(scr + kNoAllocCtl);
     sa.dq = reinterpret_cast<uint4 *>(scr + kNoAllocCtl + kNoAllocCtlWords);
     sa.dq_cap = (unsigned)kNoAllocQueue;
-    sa.spin_limit = 1u << 19;
+    if (ctx->limits.noalloc_queue > 0)
+      sa.dq_cap = std::min(sa.dq_cap, (unsigned)ctx->limits.noalloc_queue);
+    sa.spin_limit = ctx->limits.noalloc_polls > 0 ? (unsigned)ctx->limits.noalloc_polls : 1u << 19;
     stream_limits(ctx, sa);
     PJ_CK(launch_pdl(ks, std::max(1, occ_s) * ctx->num_sms, 128, ssmem, s, sa));
     int64_t blocks = std::min<int64_t>((int64_t)occ * ctx->num_sms, (n * 32 + threads - 1) / threads);

@@ -200,6 +200,7 @@ pj_status run_join_tiled(Ctx *ctx, const pj_host_meshes *Am, const pj_host_meshe
   int direct = 0;
   PJ_CK(cudaDeviceGetAttribute(&direct, cudaDevAttrPageableMemoryAccessUsesHostPageTables,
                                ctx->device));
+  if (ctx->limits.tiled_host_gather) direct = 0;
   HostSet A, B;
   pj_status st;
   if ((st = prepare(ctx, Am, W, L, direct != 0, A)) != PJ_OK) return st;

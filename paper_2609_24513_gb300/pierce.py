@@ -158,6 +158,11 @@ class pj_tiled_stats(ctypes.Structure):
                 ("ms_device", ctypes.c_float), ("reserved2", ctypes.c_float)]
 
 
+class pj_test_limits(ctypes.Structure):
+    _fields_ = [("noalloc_polls", ctypes.c_int32), ("noalloc_queue", ctypes.c_int32),
+                ("tiled_host_gather", ctypes.c_int32), ("reserved", ctypes.c_int32)]
+
+
 # pj_dsjoin_opts.materialize (the paper's strategies, Sec. 3.5)
 PJ_MAT_ESTIMATED, PJ_MAT_TWO_PASS, PJ_MAT_FIXED = range(3)
 MATERIALIZE = {"estimated": 0, "two_pass": 1, "fixed": 2}
@@ -197,6 +202,7 @@ SIGNATURES = {
                        ctypes.POINTER(pj_query_stats)]),
     "pj_get_counters": (_i32, [_vp, ctypes.POINTER(pj_counters)]),
     "pj_reset_counters": (_i32, [_vp]),
+    "pj_set_test_limits": (_i32, [_vp, ctypes.POINTER(pj_test_limits)]),
     "pj_segtri_batch": (_i32, [_vp, _vp, _vp, _i64, _i32, _vp, ctypes.POINTER(_i64), _vp]),
     "pj_export_bvh": (_i32, [_vp, _i32, _i32, _i32, _vp, _vp, _vp, ctypes.POINTER(_i64)]),
     "pj_export_mesh_data": (_i32, [_vp, _i32, _vp, _vp, _vp]),
@@ -503,6 +509,11 @@ def pj_get_counters(ctx) -> dict:
 
 def pj_reset_counters(ctx):
     _check(ctx, load().pj_reset_counters(ctx))
+
+
+def pj_set_test_limits(ctx, **limits):
+    """Limits of a context for tests (fields of pj_test_limits; none: reset)."""
+    _check(ctx, load().pj_set_test_limits(ctx, ctypes.byref(pj_test_limits(**limits))))
 
 
 def pj_segtri_batch(ctx, pq, abc, res, mode=PJ_LEAF_FILTERED, stream=None) -> int:

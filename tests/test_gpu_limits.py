@@ -1,0 +1,93 @@
+"""Paths that ordinary sizes do not reach, brought within reach of small data by
+a context's test limits: the allocation-free join whose waits run out or whose
+task queue fills (its launch behind then redoes every pair, and the next call
+clears the queue), and the tiled join with the host gathering the cells.  All
+against the oracle."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2609_24513_gb300 import pierce, synth
+from test_gpu_join import _bipyramid
+from test_zz_no_alloc import _noalloc
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = pierce.Context(0)
+    yield c
+    c.close()
+
+
+@pytest.fixture(scope="module")
+def dense():
+    # bipyramids: nearly all their node pairs overlap, so that stacks fill
+    m, tw = (_bipyramid(300, (0.5, 0.5, 0.5), 0.2, 0.2, phase=p) for p in (0.0, 0.5))
+    A, B = synth.concat([m, m, tw]), synth.concat([m, tw, synth.translate(m, (1.0, 0.0, 0.0))])
+    cand = np.array([(i, j) for i in range(3) for j in range(3)], np.int32)
+    truth = oracle.join(A, B, cand, tier=2).astype(bool)
+    return A, B, np.tile(cand, (40, 1)), np.tile(truth, 40)
+
+
+@pytest.mark.parametrize("W,L", [(2, 1), (4, 2), (8, 1)])
+@pytest.mark.parametrize("limits", [dict(noalloc_polls=1), dict(noalloc_queue=1),
+                                    dict(noalloc_queue=40), dict(noalloc_queue=2000)])
+def test_noalloc_join_that_fails_over(ctx, dense, W, L, limits):
+    torch = pytest.importorskip("torch")
+    A, B, cand, truth = dense
+    assert truth.any() and not truth.all()
+    ha, hb = ctx.load(A), ctx.load(B)
+    ctx.build(ha, W, L)
+    ctx.build(hb, W, L)
+
+    def call():
+        before = ctx.counters()["pairs_refined"]
+        k, pairs, flags = _noalloc(ctx, ha, hb, cand, torch)
+        assert np.array_equal(flags.astype(bool), truth)
+        assert k == int(truth.sum()) and np.array_equal(pairs, cand[truth])
+        return ctx.counters()["pairs_refined"] - before
+
+    assert call() == len(cand)            # the streaming launch did it
+    for _ in range(2):                    # the limit, then a call without it
+        pierce.pj_set_test_limits(ctx.h, **limits)
+        refined = [call() for _ in range(2)]
+        pierce.pj_set_test_limits(ctx.h)
+        if limits.get("noalloc_polls") or limits.get("noalloc_queue") == 1:
+            assert min(refined) > len(cand)   # the launch behind it redid the pairs
+        assert call() == len(cand)
+    pierce.pj_free_dataset(ctx.h, ha)
+    pierce.pj_free_dataset(ctx.h, hb)
+
+
+@pytest.mark.parametrize("grid", [1, 2, 3])
+def test_tiled_join_gathered_by_the_host(ctx, grid):
+    A, B = synth.tiny_spheres(1003)
+    U = synth.urban(5001, n_buildings=400, n_parts=40)
+    want, want_u = oracle.join_all(A, B), oracle.join_all(U, U, self_join=True)
+    cut = synth.MeshSet(A.xyz, A.tris, A.voff[3:], A.toff[3:])
+    for host in (1, 0):
+        pierce.pj_set_test_limits(ctx.h, tiled_host_gather=host)
+        got, st = pierce.pj_join_tiled(ctx.h, A, B, grid=grid)
+        assert np.array_equal(got, want) and st["grid"] == grid
+        got, _ = pierce.pj_join_tiled(ctx.h, U, self_join=True, grid=grid)
+        assert np.array_equal(got, want_u)
+        got, _ = pierce.pj_join_tiled(ctx.h, cut, B, grid=grid)
+        assert np.array_equal(got, want[want[:, 0] >= 3] - [3, 0])
+        if host:
+            assert st["ms_gather"] > 0    # it was the host
+    bad = synth.MeshSet(A.xyz.copy(), A.tris, A.voff, A.toff)
+    bad.xyz[5, 1] += 0.5
+    for host in (1, 0):
+        pierce.pj_set_test_limits(ctx.h, tiled_host_gather=host)
+        with pytest.raises(pierce.PierceError) as e:
+            pierce.pj_join_tiled(ctx.h, bad, B, grid=grid)
+        assert e.value.code == 2          # PJ_ERR_NOT_QUANTIZED
+    pierce.pj_set_test_limits(ctx.h)
+
+
+def test_limits_refuse_no_context():
+    assert pierce.load().pj_set_test_limits(None, ctypes.byref(pierce.pj_test_limits())) == 1
