@@ -646,7 +646,8 @@ typedef struct {
   int32_t noalloc_queue;    /* and entries of its task queue that it uses    */
   int32_t tiled_host_gather; /* 1: pj_join_tiled works out boxes and gathers
                                cells on the host even where the device can    */
-  int32_t reserved;
+  int32_t parity_list;      /* joins: entries of the list of parity rays that
+                               threads hand to warps                          */
 } pj_test_limits;
 
 /* Set a context's test limits (NULL: none). */

@@ -1142,6 +1142,8 @@ pj_status pj_set_test_limits(pj_ctx *h, const pj_test_limits *limits) {
   if (!ctx) return PJ_ERR_INVALID_ARG;
   std::lock_guard<std::mutex> lk(ctx->mu);
   ctx->limits = limits ? *limits : pj_test_limits{};
+  for (auto &g : ctx->graphs) cudaGraphExecDestroy(g.second);  // captured with the old ones
+  ctx->graphs.clear();
   return PJ_OK;
 }
 

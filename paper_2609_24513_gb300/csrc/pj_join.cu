@@ -1161,6 +1161,10 @@ struct WaveArgs {
   uint4 *q_par;              // parity rays over the per-thread node budget
   unsigned int *q_par_n;
   unsigned int q_par_cap;
+  // searches past surface vertices (see hand_surface): those handed over, the
+  // resident warps, the most that may be
+  unsigned int *q_surf_n;
+  unsigned int q_surf_warps, q_surf_cap;
   int par_dirs;              // parity rays cast: bit 0 inside(B, A), bit 1 inside(A, B)
   uint8_t *pflags;           // where parity results go (null: flags)
   const uint8_t *need;       // non-null: only candidates with need[c] != 0 are traversed
@@ -1511,7 +1515,7 @@ __global__ void __launch_bounds__(256, 3) k_wave_leaf(WaveArgs P, const uint4 *l
 // threads, inside(A, B) for odd ones.  Depth-first with a per-thread stack
 // (bounded by 1 + (W - 1) * depth).  A ray that needs more than
 // kParNodeBudget nodes (one that runs along a long tube, say) would hold its
-// whole block back; it is handed to the warp passes instead (-2).
+// whole block back; it is handed to a warp instead (-2).
 constexpr int kParNodeBudget = 4;
 constexpr uint32_t kParItem = 0xFFFFFFFEu;  // queue entry: (c, kParItem, direction)
 
@@ -1575,6 +1579,31 @@ __device__ int thread_parity(const Side &T, int it, int64_t tbase, F3 toff, F3 v
   return par | (on ? 2 : 0);
 }
 
+__device__ __forceinline__ unsigned ld_vol(const unsigned *p) {
+  return *reinterpret_cast<volatile const unsigned *>(p);
+}
+
+// A vertex on the other surface decides nothing: the next one is looked at.  A
+// warp tests 32 of them at once, but its turn costs as much as about eight of
+// a thread's vertices, and the warps take theirs one after another.  So after
+// its k-th such vertex the thread hands the direction over if fewer than
+// 1 + k / 8 of them per resident warp have been, and from kSurfMost vertices
+// on in any case, as far as their share of the list goes; otherwise it casts
+// the next vertex's ray.  Few or long searches (the walls of the urban self
+// join: 91 us of parity without the list, 47 with it) thus go to warps, and
+// lists of many short ones stay with the threads: a join of 1,000,000 boxes
+// against boxes that share a face takes 1.19 ms, 2.60 with every one handed
+// over and 1.13 with none (20,000 tessellated towers on themselves: 16.7 ms,
+// 16.7 and 263).
+constexpr int kSurfMost = 64;
+
+__device__ __forceinline__ bool hand_surface(const WaveArgs &P, int k) {
+  const unsigned most = k >= kSurfMost ? P.q_surf_cap
+                                       : min(P.q_surf_cap, P.q_surf_warps * (1u + (unsigned)k / 8u));
+  // (read first: the claims of a long list would queue up)
+  return ld_vol(P.q_surf_n) < most && atomicAdd(P.q_surf_n, 1u) < most;
+}
+
 template <int W>
 __global__ void __launch_bounds__(128) k_wave_parity(WaveArgs P) {
   pdl_wait();
@@ -1592,9 +1621,15 @@ __global__ void __launch_bounds__(128) k_wave_parity(WaveArgs P) {
   int gap = 1;
   while (gap < 32 && n * gap * 2 <= stride) gap *= 2;
   const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  for (int64_t g = tid % gap ? n : tid / gap; g < n; g += stride) {
+  // one vertex of a direction at a time: only the direction and the vertex's
+  // number stay in registers between rays
+  int64_t g = tid % gap ? n : tid / gap;
+  for (int k = 0; g < n;) {
     const int64_t c = g >> 1;
     const bool bInA = (g & 1) == 0;
+    const int kk = k;  // (the next direction's first, unless this one goes on)
+    k = 0;
+    g += stride;
     if (!((P.par_dirs >> (bInA ? 0 : 1)) & 1)) continue;  // direction not asked for
     const int ia = P.cand[2 * c], ib = P.cand[2 * c + 1];
     if (ia < 0 || ia >= P.MA || ib < 0 || ib >= P.MB) continue;
@@ -1610,11 +1645,17 @@ __global__ void __launch_bounds__(128) k_wave_parity(WaveArgs P) {
     const float4 q0 = Q.mrec[3 * (int64_t)iq], q1 = Q.mrec[3 * (int64_t)iq + 1];
     const float4 q2 = Q.mrec[3 * (int64_t)iq + 2];
     const int64_t tbase = __float_as_int(t2.y);
-    const int nv = __float_as_int(q2.w);
     const F3 lo = add(mkf3(t0.x, t0.y, t0.z), toff), hi = add(mkf3(t1.x, t1.y, t1.z), toff);
-    bytes += 96;
-    if (nv <= 0) continue;
-    const F3 v = add(mkf3(q0.w, q1.w, q2.x), qoff);
+    if (kk >= __float_as_int(q2.w)) continue;  // no (further) vertex
+    F3 v;
+    if (kk == 0) {
+      v = mkf3(q0.w, q1.w, q2.x);
+      bytes += 96;
+    } else {
+      v = ld3(Q.xyz + 3 * (int64_t)Q.lexorder[(int64_t)__float_as_int(q2.z) + kk]);
+      bytes += 16;
+    }
+    v = add(v, qoff);
     if (v.x < lo.x || v.x > hi.x || v.y < lo.y || v.y > hi.y || v.z < lo.z || v.z > hi.z) continue;
     rays += 1;
     const unsigned long long n0 = nodes, tr0 = tris;
@@ -1622,17 +1663,25 @@ __global__ void __launch_bounds__(128) k_wave_parity(WaveArgs P) {
     ray_axis_choice(v, lo, hi, ax, dir);
     const int r = thread_parity<W>(T, it, tbase, toff, v, ax, dir, stk, CAP, nodes, tris);
     bytes += (nodes - n0) * W * 32 + (tris - tr0) * 48;
-    if (r == -2 || (r >= 0 && (r & 2))) {
-      // over the node budget, or the vertex lies on T's surface and others
-      // have to be looked at: a warp redoes this direction from the start (it
-      // looks at 32 vertices at once; the thread took them one after another,
-      // 91 us on the urban self join against 47)
-      handed += 1;
+    const bool on = r >= 0 && (r & 2);
+    if (r == -2 || (on && hand_surface(P, kk))) {
+      // a warp redoes this direction from the start
       const unsigned pos = atomicAdd(P.q_par_n, 1u);
-      if (pos < P.q_par_cap) P.q_par[pos] = make_uint4((uint32_t)c, kParItem, bInA ? 0u : 1u, 0u);
-      else atomicCAS(P.err, 0, DERR_QUEUE);
-    } else if (r < 0) {
+      if (pos < P.q_par_cap) {
+        handed += 1;
+        P.q_par[pos] = make_uint4((uint32_t)c, kParItem, bInA ? 0u : 1u, 0u);
+        continue;
+      }
+      if (r == -2) {
+        atomicCAS(P.err, 0, DERR_QUEUE);
+        continue;
+      }
+    }
+    if (r < 0) {
       atomicCAS(P.err, 0, DERR_STACK);
+    } else if (on) {
+      g -= stride;
+      k = kk + 1;
     } else if (r & 1) {
       (P.pflags ? P.pflags : P.flags)[c] = 1;
     }
@@ -1912,10 +1961,6 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
-}
-
-__device__ __forceinline__ unsigned ld_vol(const unsigned *p) {
-  return *reinterpret_cast<volatile const unsigned *>(p);
 }
 
 // A queue entry's ready word: 1 for a traversal task (candidate, item A,
@@ -3285,8 +3330,13 @@ pj_status run_join(Ctx *ctx, Dataset *A, Dataset *B, const int32_t *cand,
   // first warp pass in the last queue and the parity hand-over count/position
   unsigned int *wctr = nullptr;
   const int wctr_words = 2 * std::max(wave_levels, 0) + SQ_WORDS + 8;
-  const unsigned int wpar_cap =
-      (unsigned int)std::min<int64_t>(std::max<int64_t>(2 * Ccap, 1024), 1 << 22);
+  // the list of parity rays handed to warps: an entry a direction, at most 100
+  // MB.  Where that is not one for each, a quarter is for searches past
+  // surface vertices, which threads can also end themselves; the rest stays
+  // for the rays over the node budget, which they cannot
+  const int64_t wpar_all = std::max<int64_t>(2 * Ccap, 1024);
+  const unsigned int wpar_cap = (unsigned int)std::min<int64_t>(
+      wpar_all, ctx->limits.parity_list > 0 ? ctx->limits.parity_list : 3 << 21);
   int wave_grid[3] = {1, 1, 1};  // expand/init, leaf, parity: one resident wave
   bool front = (wave_levels > 0 || stream) && o->launch_mode != PJ_LAUNCH_PER_PAIR;
   int stream_grid = 1, stream_smem = 0;
@@ -3415,6 +3465,9 @@ pj_status run_join(Ctx *ctx, Dataset *A, Dataset *B, const int32_t *cand,
     wa.q_par = wpar;
     wa.q_par_n = nullptr;
     wa.q_par_cap = wpar_cap;
+    wa.q_surf_n = nullptr;
+    wa.q_surf_cap = wpar_all <= (int64_t)wpar_cap ? wpar_cap : wpar_cap / 4;
+    wa.q_surf_warps = 16u * (unsigned)ctx->num_sms;
     wa.par_dirs = pred == PJ_PRED_OVERLAP ? 0 : (pred == PJ_PRED_CONTAINS ? 1 : (pred == PJ_PRED_WITHIN ? 2 : 3));
     wa.pflags = d_pflags;
     wa.need = d_pflags;  // contains / within: traverse where the parity test holds
@@ -3452,6 +3505,7 @@ pj_status run_join(Ctx *ctx, Dataset *A, Dataset *B, const int32_t *cand,
         // intake position of a hand-over launch
         unsigned int *sc = wctr, *hc = wctr + SQ_WORDS;
         wa.q_par_n = hc;
+        wa.q_surf_n = hc + 4;
         // the long rays go to warps before the traversal: a containment-only
         // pair (no crossing to stop at) is the costliest kind to traverse.
         // (Running the parity launches on a second stream beside the
@@ -3506,7 +3560,7 @@ pj_status run_join(Ctx *ctx, Dataset *A, Dataset *B, const int32_t *cand,
         WaveArgs wa = make_wave_args();
         unsigned int *qn = wctr, *ln = wctr + wave_levels + 1, *misc = ln + wave_levels;
         wa.q_par_n = misc + 1;
-        wa.q_par_cap = wpar_cap;
+        wa.q_surf_n = misc + 5;
         WaveExpandKernel kx = pick_wave_expand(W);
         WaveLeafKernel kl = pick_wave_leaf(W, exact);
         WaveParityKernel kp = pick_wave_parity(W);

@@ -1,8 +1,8 @@
 """Paths that ordinary sizes do not reach, brought within reach of small data by
 a context's test limits: the allocation-free join whose waits run out or whose
 task queue fills (its launch behind then redoes every pair, and the next call
-clears the queue), and the tiled join with the host gathering the cells.  All
-against the oracle."""
+clears the queue), joins whose list of handed-over parity rays fills, and the
+tiled join with the host gathering the cells.  All against the oracle."""
 import ctypes
 
 import numpy as np
@@ -30,7 +30,7 @@ def dense():
     A, B = synth.concat([m, m, tw]), synth.concat([m, tw, synth.translate(m, (1.0, 0.0, 0.0))])
     cand = np.array([(i, j) for i in range(3) for j in range(3)], np.int32)
     truth = oracle.join(A, B, cand, tier=2).astype(bool)
-    return A, B, np.tile(cand, (40, 1)), np.tile(truth, 40)
+    return A, B, np.tile(cand, (4, 1)), np.tile(truth, 4)
 
 
 @pytest.mark.parametrize("W,L", [(2, 1), (4, 2), (8, 1)])
@@ -59,6 +59,64 @@ def test_noalloc_join_that_fails_over(ctx, dense, W, L, limits):
         if limits.get("noalloc_polls") or limits.get("noalloc_queue") == 1:
             assert min(refined) > len(cand)   # the launch behind it redid the pairs
         assert call() == len(cand)
+    pierce.pj_free_dataset(ctx.h, ha)
+    pierce.pj_free_dataset(ctx.h, hb)
+
+
+def test_touching_boxes_beyond_the_parity_list(ctx):
+    # the same two boxes 2,200,000 times: both directions' first vertices lie on
+    # the other's surface, more directions than 2^22.  Threads look at further
+    # vertices themselves, so that nothing is redone
+    box = synth.concat([synth.box((1000, 1000, 1000), (9000, 9000, 9000))])
+    ha, hb = ctx.load(box), ctx.load(box)
+    ctx.build(ha, 4, 2)
+    ctx.build(hb, 4, 2)
+    launches = []
+    for n in (2000, 2200000):
+        before = ctx.counters()["kernel_launches"]
+        got, info = ctx.join(ha, hb, cand=np.zeros((n, 2), np.int32))
+        assert info["n_candidates"] == n and len(got) == 0      # identical meshes
+        launches.append(ctx.counters()["kernel_launches"] - before)
+    assert launches[0] == launches[1]
+    pierce.pj_free_dataset(ctx.h, ha)
+    pierce.pj_free_dataset(ctx.h, hb)
+
+
+@pytest.fixture(scope="module")
+def walls():
+    # towers of 8 to 441 wall vertices against neighbours that share the wall,
+    # stand inside against it, are the same, or touch in an edge
+    sets = []
+    for per, bands in ((1, 1), (2, 1), (3, 2), (4, 15), (20, 20)):
+        foot = np.rint(synth._rect(8000, 8000, per) + 50000)
+        t = synth.building(foot, 1000, 8000, 100, bands)
+        sets.append((t, [synth.translate(t, (8000, 0, 0)), t, synth.translate(t, (8000, 8000, 0)),
+                         synth.box((46000, 47000, 2000), (48000, 51000, 6000))]))
+    A = synth.concat([t for t, _ in sets])
+    B = synth.concat([m for _, ms in sets for m in ms])
+    cand = np.array([(i, 4 * i + k) for i in range(len(sets)) for k in range(4)], np.int32)
+    return A, B, cand, {p: oracle.join(A, B, cand, predicate=p).astype(bool)
+                        for p in ("intersects", "contains", "within")}
+
+
+@pytest.mark.parametrize("limit", [0, 1, 7, 64])
+@pytest.mark.parametrize("W,L,levels", [(2, 1, 0), (4, 2, 0), (8, 4, 0), (4, 2, 4)])
+def test_surface_vertices_over_parity_list_sizes(ctx, walls, limit, W, L, levels):
+    # no limit: the first directions go to warps, then those past 8, 16, ...
+    # vertices; small lists: threads go on to the last vertex
+    A, B, cand, truth = walls
+    assert truth["intersects"].any() and truth["contains"].any()
+    ha, hb = ctx.load(A), ctx.load(B)
+    ctx.build(ha, W, L)
+    ctx.build(hb, W, L)
+    pierce.pj_set_test_limits(ctx.h, parity_list=limit)
+    for reps in (1, 1500):
+        c = np.tile(cand, (reps, 1))
+        for pred, t in truth.items():
+            got, _ = ctx.join(ha, hb, cand=c, width=W, leaf_size=L, predicate=pred,
+                              wave_levels=levels)
+            assert np.array_equal(got, c[np.tile(t, reps)]), (pred, reps)
+    pierce.pj_set_test_limits(ctx.h)
     pierce.pj_free_dataset(ctx.h, ha)
     pierce.pj_free_dataset(ctx.h, hb)
 
