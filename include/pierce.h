@@ -328,7 +328,7 @@ pj_status pj_free_pairs(pj_ctx *ctx, pj_pairs *res);
  * *d_count -1; the next call clears that state.  Asynchronous: the work is enqueued on cuda_stream (NULL: the
  * context's stream) and the outputs are valid once it has completed.
  * n_cand above 16,777,216 is rejected with PJ_ERR_INVALID_ARG.
- * Scratch: a 2,163,520-byte array in device global memory, defined at file
+ * Scratch: a 16,843,584-byte array in device global memory, defined at file
  * scope in the library; every GPU that loads the library holds it until the
  * process exits.  The first call on a device looks up the array's device
  * address (make that first call before any stream capture).  All calls on a

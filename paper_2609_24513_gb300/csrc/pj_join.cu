@@ -3878,7 +3878,7 @@ pj_status run_join(Ctx *ctx, Dataset *A, Dataset *B, const int32_t *cand,
 // buffers for the candidates, the per-candidate flags, the pairs and the
 // count; the scratch the kernels need (candidate count, work counters, error
 // words, per-chunk counts and offsets of the compaction, the streaming
-// kernel's control words and task queue: 2.1 MB) lives in one file-scope
+// kernel's control words and task queue: 16.8 MB) lives in one file-scope
 // device array shared by every call on a device.
 //
 // The refinement is the streaming kernel's.  A warp per pair in plain
@@ -3887,10 +3887,17 @@ pj_status run_join(Ctx *ctx, Dataset *A, Dataset *B, const int32_t *cand,
 // ---------------------------------------------------------------------------
 constexpr int64_t kNoAllocMaxChunks = 4096;
 constexpr int64_t kNoAllocMaxCand = kNoAllocMaxChunks * CMP_CHUNK;  // 16,777,216
-// the streaming launch's task queue (each entry is used once a launch: a
-// join of 1,501 x 75 tissue meshes puts about 15,000 through it; when it is
-// full the warps keep their work)
-constexpr int64_t kNoAllocQueue = 131072;
+// The streaming launch's task queue; each entry is used once a launch.  Tasks
+// go through it when warps run out of candidates, so what it takes follows the
+// costly end of a list more than its length: 10,000 x 500 tissue meshes 94,000
+// (W = 8, L = 8) to 191,000 (W = 2, L = 2), the same list 16 times over
+// 186,000 (W = 4, L = 2).  When it is full the warps keep their work, and one
+// whose stack is full then fails the launch.  With 131,072 entries, which
+// most of those fill, they took 834 us (W = 4, L = 2) and 1,114 (W = 2), 407
+// and 486 now; 300 pairs of 2,000-triangle bipyramids, nearly all of whose
+// nodes meet, failed then (1,010 ms) and put 343,000-845,000 entries through
+// it now (18-30 ms).
+constexpr int64_t kNoAllocQueue = 1 << 20;
 // int64 words: [0] candidate count, [1] work counter of the fallback, [2..3]
 // four int error words, [4] work counter of the parity pass, [5] the
 // streaming launch's error word, [6..7] unused, then kNoAllocMaxChunks chunk

@@ -121,6 +121,27 @@ def test_surface_vertices_over_parity_list_sizes(ctx, walls, limit, W, L, levels
     pierce.pj_free_dataset(ctx.h, hb)
 
 
+def test_noalloc_join_of_the_full_tissue(ctx, pathology_truth):
+    # more tasks change hands than a queue of 131,072 entries took, and all of
+    # them fit
+    torch = pytest.importorskip("torch")
+    A, B, cand, truth = pathology_truth
+    truth = truth.astype(bool)
+    ha, hb = ctx.load(A), ctx.load(B)
+    ctx.build(ha, 2, 2)
+    ctx.build(hb, 2, 2)
+    for _ in range(2):
+        ctx.reset_counters()
+        k, pairs, flags = _noalloc(ctx, ha, hb, cand, torch)
+        assert np.array_equal(flags.astype(bool), truth)
+        assert k == int(truth.sum()) and np.array_equal(pairs, cand[truth])
+        c = ctx.counters()
+        assert c["pairs_refined"] == len(cand)            # nothing was redone
+        assert 131072 < c["tasks_spilled"] < 1 << 20
+    pierce.pj_free_dataset(ctx.h, ha)
+    pierce.pj_free_dataset(ctx.h, hb)
+
+
 @pytest.mark.parametrize("grid", [1, 2, 3])
 def test_tiled_join_gathered_by_the_host(ctx, grid):
     A, B = synth.tiny_spheres(1003)
