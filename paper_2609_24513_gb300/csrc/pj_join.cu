@@ -3942,8 +3942,8 @@ __global__ void __launch_bounds__(256) k_noalloc_begin(int64_t *scr, int64_t n) 
   scr[4] = 0;  // work counter of the parity pass
 }
 
-// Containment of the allocation-free join, before its streaming launch: all
-// flags cleared, then one warp per (candidate, direction) whose
+// The allocation-free join before its streaming launch: candidate ids checked,
+// all flags cleared, and containment: one warp per (candidate, direction) whose
 // representative vertex lies in the other mesh's box; 1 where it is inside.
 // (The per-thread parity kernel of the other joins hands its long rays over
 // through a list sized by the candidates, which this entry point has no room
@@ -3952,6 +3952,8 @@ __global__ void __launch_bounds__(256) k_noalloc_begin(int64_t *scr, int64_t n) 
 // outgrow the stack is repeated in plain depth-first order, which fits.
 template <int W>
 __global__ void __launch_bounds__(128, 4) k_pair_parity(RefineArgs P, int64_t *stream_err) {
+  pdl_wait();
+  pdl_trigger();
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   if (blockIdx.x == 0 && threadIdx.x == 0) *stream_err = 0;
@@ -3979,6 +3981,8 @@ __global__ void __launch_bounds__(128, 4) k_pair_parity(RefineArgs P, int64_t *s
                 b2.x <= a1.z) |
                (a0.w >= b0.x && a0.w <= b1.x && a1.w >= b0.y && a1.w <= b1.y && a2.x >= b0.z &&
                 a2.x <= b1.z) << 1;
+      } else {
+        atomicCAS(P.err + 1, 0, 1);
       }
     }
     __syncwarp();  // the flags are cleared before any is set
@@ -4014,6 +4018,8 @@ static PairParityKernel pick_pair_parity(int W) {
 // pair count (-1 if a device-side check failed)
 __global__ void k_noalloc_scan(const int64_t *counts, int64_t *offs, int64_t nchunks,
                                const int *err, int64_t *out_count) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ int64_t carry;
   if (threadIdx.x == 0) carry = 0;
   __syncthreads();
@@ -4106,16 +4112,14 @@ pj_status run_join_noalloc(Ctx *ctx, Dataset *A, Dataset *B, const int32_t *d_ca
 
   k_noalloc_begin<<<64, 256, 0, s>>>(scr, n);
   if (n > 0) {
-    k_check_cand<<<std::min(blocks_for(n, 256), ctx->num_sms * 8), 256, 0, s>>>(
-        d_cand, nullptr, n, A->M, B->M, B->d_aabb, err, nullptr, nullptr);
     const PairParityKernel kp = pick_pair_parity(W);
     int occ_p = 0;
     PJ_CK(occupancy(ctx->device, (const void *)kp, threads, smem, &occ_p));
     RefineArgs pa = args;
     pa.work = reinterpret_cast<unsigned long long *>(scr + 4);
     const int64_t most = (n + threads / 32 - 1) / (threads / 32);
-    kp<<<(int)std::min<int64_t>((int64_t)std::max(occ_p, 1) * ctx->num_sms, most), threads, smem, s>>>(
-        pa, scr + 5);
+    PJ_CK(launch_pdl(kp, (int)std::min<int64_t>((int64_t)std::max(occ_p, 1) * ctx->num_sms, most),
+                     threads, smem, s, pa, scr + 5));
     const StreamKernel ks = pick_stream(W, false);
     const int ssmem = 4 * stream_smem_per_warp(W);
     int occ_s = 0;
@@ -4141,12 +4145,15 @@ pj_status run_join_noalloc(Ctx *ctx, Dataset *A, Dataset *B, const int32_t *d_ca
     stream_limits(ctx, sa);
     PJ_CK(launch_pdl(ks, std::max(1, occ_s) * ctx->num_sms, 128, ssmem, s, sa));
     int64_t blocks = std::min<int64_t>((int64_t)occ * ctx->num_sms, (n * 32 + threads - 1) / threads);
-    kern<<<(int)std::max<int64_t>(blocks, 1), threads, smem, s>>>(args);
+    PJ_CK(launch_pdl(kern, (int)std::max<int64_t>(blocks, 1), threads, smem, s, args));
   }
   const int nchunks = (int)std::max<int64_t>(1, (n + CMP_CHUNK - 1) / CMP_CHUNK);
-  k_flag_count<<<nchunks, CMP_T, 0, s>>>(d_flags, d_n, counts, ctx->d_counters + C_HITS);
-  k_noalloc_scan<<<1, SCAN_T, 0, s>>>(counts, offs, nchunks, err, d_count);
-  k_flag_emit<<<nchunks, CMP_T, 0, s>>>(d_flags, d_n, d_cand, offs, d_pairs);
+  PJ_CK(launch_pdl(k_flag_count, nchunks, CMP_T, 0, s, (const uint8_t *)d_flags,
+                   (const int64_t *)d_n, counts, ctx->d_counters + C_HITS));
+  PJ_CK(launch_pdl(k_noalloc_scan, 1, SCAN_T, 0, s, (const int64_t *)counts, offs,
+                   (int64_t)nchunks, (const int *)err, d_count));
+  PJ_CK(launch_pdl(k_flag_emit, nchunks, CMP_T, 0, s, (const uint8_t *)d_flags,
+                   (const int64_t *)d_n, d_cand, (const int64_t *)offs, d_pairs));
   PJ_CK(cudaGetLastError());
   return PJ_OK;
 }

@@ -121,6 +121,47 @@ def test_surface_vertices_over_parity_list_sizes(ctx, walls, limit, W, L, levels
     pierce.pj_free_dataset(ctx.h, hb)
 
 
+@pytest.mark.parametrize("n", [1, 31, 400, 90000])
+def test_noalloc_join_finds_bad_ids_and_replays(ctx, n):
+    # ids out of range anywhere in a warp's share; then the queued launches
+    # captured once and replayed over other candidates
+    torch = pytest.importorskip("torch")
+    A, B = synth.tiny_spheres(1001)
+    every = np.array([(i, j) for i in range(A.nmesh) for j in range(B.nmesh)], np.int32)
+    truth = oracle.join(A, B, every, tier=2).astype(bool)
+    rng = np.random.default_rng(n)
+    pick = rng.integers(0, len(every), size=n)
+    ha, hb = ctx.load(A), ctx.load(B)
+    ctx.build(ha, 4, 2)
+    ctx.build(hb, 4, 2)
+    for at, bad in ((0, (A.nmesh, 0)), (n - 1, (0, B.nmesh)), (n // 2, (-1, 0)), (n // 3, (0, -1))):
+        cand = every[pick]
+        cand[at] = bad
+        k, _, flags = _noalloc(ctx, ha, hb, cand, torch)
+        want = truth[pick].copy()
+        want[at] = False
+        assert k == -1 and np.array_equal(flags.astype(bool), want)
+    d_cand = torch.from_numpy(every[pick]).cuda()
+    d_flags = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    d_pairs = torch.zeros((n, 2), dtype=torch.int32, device="cuda")
+    d_count = torch.zeros(1, dtype=torch.int64, device="cuda")
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        pierce.pj_join_intersects_noalloc(ctx.h, ha, hb, d_cand, d_flags, d_pairs, d_count,
+                                          stream=torch.cuda.current_stream())
+    for _ in range(3):
+        pick = rng.integers(0, len(every), size=n)
+        d_cand.copy_(torch.from_numpy(every[pick]))
+        g.replay()
+        torch.cuda.synchronize()
+        t = truth[pick]
+        assert int(d_count.item()) == t.sum()
+        assert np.array_equal(d_flags.cpu().numpy().astype(bool), t)
+        assert np.array_equal(d_pairs[:int(t.sum())].cpu().numpy(), every[pick][t])
+    pierce.pj_free_dataset(ctx.h, ha)
+    pierce.pj_free_dataset(ctx.h, hb)
+
+
 def test_noalloc_join_of_the_full_tissue(ctx, pathology_truth):
     # more tasks change hands than a queue of 131,072 entries took, and all of
     # them fit
