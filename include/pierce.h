@@ -360,7 +360,8 @@ typedef struct {
 
 typedef struct {
   int64_t device_budget;    /* device bytes one cell's meshes and BVHs may
-                               take (0: a quarter of the free memory)        */
+                               take (0: a quarter of the free memory, unused
+                               memory that the context keeps included)       */
   int32_t grid;             /* cells per axis (0: the smallest power of two,
                                at most 16, whose cells fit the budget)       */
   int32_t width;            /* per-cell BVH shape (0: 4)                     */
@@ -648,6 +649,8 @@ typedef struct {
                                cells on the host even where the device can    */
   int32_t parity_list;      /* joins: entries of the list of parity rays that
                                threads hand to warps                          */
+  int64_t tiled_free;       /* pj_join_tiled's automatic budget: the device's
+                               free bytes                                     */
 } pj_test_limits;
 
 /* Set a context's test limits (NULL: none). */

@@ -210,7 +210,13 @@ pj_status run_join_tiled(Ctx *ctx, const pj_host_meshes *Am, const pj_host_meshe
   if (budget <= 0) {
     size_t fr = 0, tot = 0;
     PJ_CK(cudaMemGetInfo(&fr, &tot));
-    budget = (int64_t)(fr / 4);
+    if (ctx->limits.tiled_free > 0) fr = (size_t)ctx->limits.tiled_free;
+    // the cells' buffers come from the context's pool: what it holds unused is
+    // as good as free
+    unsigned long long held = 0, used = 0;
+    PJ_CK(cudaMemPoolGetAttribute(ctx->mem, cudaMemPoolAttrReservedMemCurrent, &held));
+    PJ_CK(cudaMemPoolGetAttribute(ctx->mem, cudaMemPoolAttrUsedMemCurrent, &used));
+    budget = (int64_t)((fr + (held - used)) / 4);
   }
   // the grid over both datasets' box
   TGrid g;

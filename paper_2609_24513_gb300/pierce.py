@@ -160,7 +160,8 @@ class pj_tiled_stats(ctypes.Structure):
 
 class pj_test_limits(ctypes.Structure):
     _fields_ = [("noalloc_polls", ctypes.c_int32), ("noalloc_queue", ctypes.c_int32),
-                ("tiled_host_gather", ctypes.c_int32), ("parity_list", ctypes.c_int32)]
+                ("tiled_host_gather", ctypes.c_int32), ("parity_list", ctypes.c_int32),
+                ("tiled_free", ctypes.c_int64)]
 
 
 # pj_dsjoin_opts.materialize (the paper's strategies, Sec. 3.5)

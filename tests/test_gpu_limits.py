@@ -209,5 +209,25 @@ def test_tiled_join_gathered_by_the_host(ctx, grid):
     pierce.pj_set_test_limits(ctx.h)
 
 
+def test_tiled_budget_counts_memory_the_context_keeps():
+    # with almost no free memory left a tiled join still has what the context
+    # keeps of a freed dataset, and need not split its space
+    V = synth.urban(5001, n_buildings=400, n_parts=40)
+    U = synth.urban(5002, n_buildings=3000, n_parts=300)
+    want = oracle.join_all(V, V, self_join=True)
+    with pierce.Context(0) as c:
+        pierce.pj_set_test_limits(c.h, tiled_free=4096)
+        got, st = pierce.pj_join_tiled(c.h, V, self_join=True)
+        assert np.array_equal(got, want) and st["grid"] > 1
+        h = c.load(U)
+        c.build(h, 4, 2)
+        pierce.pj_free_dataset(c.h, h)
+        got, st = pierce.pj_join_tiled(c.h, V, self_join=True)
+        assert np.array_equal(got, want) and st["grid"] == 1
+        with pytest.raises(pierce.PierceError) as e:          # a given budget is kept
+            pierce.pj_join_tiled(c.h, V, self_join=True, device_budget=4096)
+        assert e.value.code == 4                              # PJ_ERR_NO_MEMORY
+
+
 def test_limits_refuse_no_context():
     assert pierce.load().pj_set_test_limits(None, ctypes.byref(pierce.pj_test_limits())) == 1
