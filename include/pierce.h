@@ -649,6 +649,9 @@ typedef struct {
                                cells on the host even where the device can    */
   int32_t parity_list;      /* joins: entries of the list of parity rays that
                                threads hand to warps                          */
+  int32_t dataset_walk;     /* pj_dataset_join: entries of the joint walk's
+                               queues and of its list of leaf pairs           */
+  int32_t reserved;
   int64_t tiled_free;       /* pj_join_tiled's automatic budget: the device's
                                free bytes                                     */
 } pj_test_limits;

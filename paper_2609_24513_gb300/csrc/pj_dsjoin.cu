@@ -493,7 +493,8 @@ template <int W>
 __global__ void __launch_bounds__(kDsLevelT) k_ds_level(const float *nodesA, const float *nodesB,
                                                         uint2 *q0, uint2 *q1, unsigned *cnt,
                                                         unsigned *at, int i, uint2 *leaves,
-                                                        unsigned *n_leaves,
+                                                        unsigned *n_leaves, unsigned queue_cap,
+                                                        unsigned leaf_cap,
                                                         unsigned long long *st) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -501,7 +502,7 @@ __global__ void __launch_bounds__(kDsLevelT) k_ds_level(const float *nodesA, con
   __shared__ uint2 s_buf[kDsLevelT / 32][2][64];
   const int lane = threadIdx.x & 31;
   uint2 *buf = s_buf[threadIdx.x >> 5][0];
-  DsOut leaf_q{buf + 64, 0, leaves, n_leaves, kDsLeaves};
+  DsOut leaf_q{buf + 64, 0, leaves, n_leaves, leaf_cap};
   int lv = (int)__ldcg(at + i);
   unsigned n = __ldcg(cnt + lv);
   const bool wide = n > kDsNarrow;
@@ -522,10 +523,10 @@ __global__ void __launch_bounds__(kDsLevelT) k_ds_level(const float *nodesA, con
   const unsigned threads = wide ? gridDim.x * kDsLevelT : kDsLevelT;
   const unsigned t0 = (wide ? blockIdx.x * kDsLevelT : 0u) + threadIdx.x - lane;
   while (n > 0 && lv < kDsLevels - 1) {
-    n = min(n, kDsQueue);
+    n = min(n, queue_cap);
     visited += 2ull * n;
     const uint2 *qin = lv & 1 ? q1 : q0;
-    DsOut next_q{buf, 0, lv & 1 ? q0 : q1, cnt + lv + 1, kDsQueue};
+    DsOut next_q{buf, 0, lv & 1 ? q0 : q1, cnt + lv + 1, queue_cap};
     for (unsigned e0 = t0 / G; e0 < n; e0 += threads / G) {
       const unsigned e = e0 + lane / G;
       const uint2 x = e < n ? __ldcg(qin + e) : make_uint2(0u, 0u);
@@ -553,7 +554,8 @@ __global__ void __launch_bounds__(kDsLevelT) k_ds_level(const float *nodesA, con
 // tests that box comparisons leave are listed and run 32 at a time.  Records
 // are counted and placed per warp of the grid.
 __global__ void __launch_bounds__(32 * kDsWarps) k_ds_leaf(DsSide A, DsSide B, const uint2 *leaves,
-                                                           const unsigned *n_leaves, int lshift,
+                                                           const unsigned *n_leaves,
+                                                          unsigned leaf_cap, int lshift,
                                                            Sink sink, unsigned long long *st) {
   __shared__ unsigned s_list[kDsWarps][128 * 3];
   const unsigned full = 0xffffffffu;
@@ -562,7 +564,7 @@ __global__ void __launch_bounds__(32 * kDsWarps) k_ds_leaf(DsSide A, DsSide B, c
   unsigned *list = s_list[wib];
   const int64_t warp = blockIdx.x * (int64_t)kDsWarps + wib, nw = gridDim.x * (int64_t)kDsWarps;
   const int64_t item = sink.base + warp;
-  const unsigned n = min(*n_leaves, kDsLeaves);
+  const unsigned n = min(*n_leaves, leaf_cap);
   unsigned long long c_tris = 0, c_hits = 0;
   int64_t n_rec = 0;
   int ntest = 0;
@@ -962,6 +964,9 @@ pj_status run_dataset_join(Ctx *ctx, Dataset *A, Dataset *B, int self_join,
   // edges by the walk of both BVHs, or in packets (see k_ds_level)
   const int levels = bA->max_depth + bB->max_depth;
   bool dual = !self_join && levels + 2 < kDsLevels;
+  const unsigned walk = (unsigned)std::max(0, ctx->limits.dataset_walk);
+  const unsigned queue_cap = walk ? std::min(walk, kDsQueue) : kDsQueue;
+  const unsigned leaf_cap = walk ? std::min(walk, kDsLeaves) : kDsLeaves;
   uint2 *q0 = nullptr, *q1 = nullptr, *leaves = nullptr;
   unsigned *lv_cnt = nullptr;  // entries per level, the leaf pairs, the launches' levels
   if (dual) {
@@ -1000,11 +1005,13 @@ pj_status run_dataset_join(Ctx *ctx, Dataset *A, Dataset *B, int self_join,
         for (int l = 0; l < levels; ++l) {
           cfg.numAttrs = l > 0;
           PJ_CK(cudaLaunchKernelEx(&cfg, kl, sA.nodes, sB.nodes, q0, q1, lv_cnt,
-                                   lv_cnt + kDsLevels + 1, l, leaves, n_leaves, d_st));
+                                   lv_cnt + kDsLevels + 1, l, leaves, n_leaves, queue_cap,
+                                   leaf_cap, d_st));
         }
         ctx->launches += levels;
       }
-      k_ds_leaf<<<leaf_grid, 32 * kDsWarps, 0, s>>>(sA, sB, leaves, n_leaves, lshift, k, d_st);
+      k_ds_leaf<<<leaf_grid, 32 * kDsWarps, 0, s>>>(sA, sB, leaves, n_leaves, leaf_cap, lshift, k,
+                                                    d_st);
     } else {
       // enough warps to spread the costly packets, few enough that their
       // counters' atomics do not queue up

@@ -161,6 +161,7 @@ class pj_tiled_stats(ctypes.Structure):
 class pj_test_limits(ctypes.Structure):
     _fields_ = [("noalloc_polls", ctypes.c_int32), ("noalloc_queue", ctypes.c_int32),
                 ("tiled_host_gather", ctypes.c_int32), ("parity_list", ctypes.c_int32),
+                ("dataset_walk", ctypes.c_int32), ("reserved", ctypes.c_int32),
                 ("tiled_free", ctypes.c_int64)]
 
 

@@ -1,8 +1,9 @@
 """Paths that ordinary sizes do not reach, brought within reach of small data by
 a context's test limits: the allocation-free join whose waits run out or whose
 task queue fills (its launch behind then redoes every pair, and the next call
-clears the queue), joins whose list of handed-over parity rays fills, and the
-tiled join with the host gathering the cells.  All against the oracle."""
+clears the queue), joins whose list of handed-over parity rays fills, dataset joins that leave the
+joint walk at a queue or the list of leaf pairs, and the tiled join with the
+host gathering the cells.  All against the oracle."""
 import ctypes
 
 import numpy as np
@@ -179,6 +180,39 @@ def test_noalloc_join_of_the_full_tissue(ctx, pathology_truth):
         c = ctx.counters()
         assert c["pairs_refined"] == len(cand)            # nothing was redone
         assert 131072 < c["tasks_spilled"] < 1 << 20
+    pierce.pj_free_dataset(ctx.h, ha)
+    pierce.pj_free_dataset(ctx.h, hb)
+
+
+@pytest.mark.parametrize("W,L", [(2, 1), (4, 2), (8, 8)])
+@pytest.mark.parametrize("predicate", ["intersects", "overlap"])
+def test_dataset_join_leaves_the_walk(ctx, W, L, predicate):
+    # from limits that the first level passes to one nothing passes: either the
+    # packets do it (their launches besides) or the walk, with the same counts
+    A, B = synth.tiny_spheres(1002)
+    cand = oracle.mbb_candidates(A, B)
+    want = cand[oracle.join(A, B, cand, predicate=predicate).astype(bool)]
+    ha, hb = ctx.load(A), ctx.load(B)
+
+    def call(mat, limit):
+        pierce.pj_set_test_limits(ctx.h, dataset_walk=limit)
+        before = ctx.counters()["kernel_launches"]
+        got, st = pierce.pj_dataset_join(ctx.h, ha, hb, width=W, leaf_size=L,
+                                         predicate=predicate, materialize=mat, fixed_slots=4096)
+        assert np.array_equal(got, want)
+        return ctx.counters()["kernel_launches"] - before, st
+
+    for mat in ("estimated", "two_pass", "fixed"):
+        call(mat, 0)
+        n, st = call(mat, 0)
+        left = []
+        for limit in (1, 33, 64, 500, 3000, 20000, 1 << 20):
+            m, s2 = call(mat, limit)
+            left.append(m > n)
+            assert m == n + left[-1] * (2 if predicate == "intersects" else 1)
+            assert s2["hits"] == st["hits"] and s2["recheck_pairs"] == st["recheck_pairs"]
+        assert left[0] and not left[-1] and left == sorted(left, reverse=True)
+    pierce.pj_set_test_limits(ctx.h)
     pierce.pj_free_dataset(ctx.h, ha)
     pierce.pj_free_dataset(ctx.h, hb)
 
