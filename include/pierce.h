@@ -76,8 +76,7 @@ typedef struct {
 
 enum { PJ_LEAF_FILTERED = 0, PJ_LEAF_EXACT = 1 };
 /* pj_segtri_batch only: the FP32 filter with the static bound of the five
- * points' box (the form the streaming kernel uses, with one bound per leaf
- * pair) */
+ * points' box (the form the streaming kernel uses) */
 enum { PJ_LEAF_STATIC = 2 };
 enum { PJ_LAUNCH_PERSISTENT = 0, PJ_LAUNCH_PER_PAIR = 1 };
 enum { PJ_FRONT_NONE = -1, PJ_FRONT_STREAM = -2 };  /* pj_join_opts.wave_levels */
@@ -121,8 +120,9 @@ typedef struct {
   int32_t wave_levels;      /* refinement front end.  0 or PJ_FRONT_STREAM:
                                the streaming kernel (one persistent launch;
                                warps keep the tasks of many pairs in shared
-                               memory, stage nodes and triangles with
-                               asynchronous copies and balance the load
+                               memory, stage nodes there with asynchronous
+                               copies, read leaf triangles into registers
+                               and balance the load
                                through a device task queue).  > 0: this many
                                BVH levels breadth-first, one thread per child
                                test, then the per-warp passes.
@@ -180,7 +180,8 @@ typedef struct {
   uint64_t box_tests;           /* child-box overlap tests                      */
   uint64_t leaf_pairs;          /* (leaf, leaf) pairs tested                    */
   uint64_t edge_slab_tests;     /* segment vs leaf-box tests (slab tests; in the
-                                   streaming kernel edge-box overlap tests)     */
+                                   streaming kernel owned edges tested by their
+                                   boxes against a leaf's triangles)            */
   uint64_t segtri_tests;        /* strict segment/triangle tests                */
   uint64_t exact_fallbacks;     /* of those, decided by the int64 path          */
   uint64_t parity_rays;         /* +z parity traversals                         */
@@ -252,7 +253,11 @@ pj_status pj_load_meshes(pj_ctx *ctx, const float *xyz, int64_t n_verts,
                          const int64_t *mesh_tri_off, int64_t n_meshes,
                          int32_t ptr_is_device, pj_dataset *out);
 
-/* Free a dataset and its BVHs. */
+/* Free a dataset and its BVHs.  Waits for the device.  The context keeps up to
+ * 4 GiB of memory freed this way (and of loading's and building's temporary
+ * buffers) for its own later loads and builds, which other allocators of the
+ * process do not get until pj_destroy; an allocation of the library that fails
+ * elsewhere gives it back first. */
 pj_status pj_free_dataset(pj_ctx *ctx, pj_dataset ds);
 
 /* Build (or reuse from the cache) the per-mesh BVHs of a dataset: an LBVH
@@ -325,8 +330,9 @@ pj_status pj_free_pairs(pj_ctx *ctx, pj_pairs *res);
  * out, a launch queued behind it redoes every pair with one warp per pair and
  * plain depth-first traversal (same result, slower).
  * A candidate id out of range is skipped (its flag stays 0) and makes
- * *d_count -1; the next call clears that state.  Asynchronous: the work is enqueued on cuda_stream (NULL: the
- * context's stream) and the outputs are valid once it has completed.
+ * *d_count -1; the next call clears that state.  Asynchronous: the work is
+ * enqueued on cuda_stream (NULL: the context's stream) and the outputs are
+ * valid once it has completed.
  * n_cand above 16,777,216 is rejected with PJ_ERR_INVALID_ARG.
  * Scratch: a 16,843,584-byte array in device global memory, defined at file
  * scope in the library; every GPU that loads the library holds it until the
@@ -462,6 +468,9 @@ typedef struct {
  * box holds the vertex than it tracks, those pairs are decided by the
  * per-pair join instead, so the result equals pj_join_intersects over the
  * bounding-box candidates exactly.  self_join: a == b, pairs i < j.
+ * The context keeps its working buffers until pj_destroy: 168 MB for the walk
+ * (a join of two datasets; without room for them the edges go in packets),
+ * 16 MB for rechecked pairs, and the hashmap or records.
  * out: sorted unique pairs (free with pj_free_pairs); stats may be NULL.
  * Synchronous. */
 pj_status pj_dataset_join(pj_ctx *ctx, pj_dataset a, pj_dataset b, int32_t self_join,

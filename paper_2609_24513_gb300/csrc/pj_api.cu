@@ -695,8 +695,9 @@ pj_status load_impl(Ctx *ctx, const float *xyz, int64_t V,
   // above), a scan, a scatter and a comparison within the lists, each about
   // one pass over the triangles.  A radix sort of all half-edges by 64-bit
   // keys made sixteen, and its run count queued a million atomics: 3,050 us
-  // for 11 M triangles, 560 now (conversion included).  Lists are compared entry by entry, so
-  // with a vertex of 255 half-edges or more the sort still does it.
+  // for 11 M triangles, 560 now (conversion included).  Lists are compared
+  // entry by entry, so with a vertex of 255 half-edges or more the sort still
+  // does it.
   if (hf[4] == 0) {
     uint2 *list;
     PJ_CK(tmp.get(&list, 3 * F));

@@ -5,11 +5,12 @@
 //     per-mesh trees, run on the dataset as one mesh; each triangle record
 //     then carries its owning mesh -- the paper's triangle-to-object map);
 //   * Alg. 1 in both directions (Sec. 3.2 "Bidirectional tracing"): every
-//     owned edge of one dataset is traced as a bounded segment through the
-//     other's BVH (conservative slab test at nodes, the exact strict
-//     segment/triangle test at leaves) and every crossing is recorded -- an
-//     edge may pierce several objects, so the traversal does not stop at the
-//     first hit (the multi-hit loop of Alg. 1);
+//     owned edge of one dataset is tested against the other's triangles around
+//     it -- found by walking the two BVHs together, or (a self join, dense
+//     data) by sending packets of 32 triangles through the other BVH -- with
+//     the exact strict segment/triangle test, and every crossing is recorded:
+//     an edge may pierce several objects, so nothing stops at the first hit
+//     (the multi-hit loop of Alg. 1);
 //   * containment (Sec. 3.3-3.4): each object casts one ray from its
 //     lexicographically first vertex through the other dataset's BVH and
 //     toggles a parity bit for every object whose triangle it crosses; an
@@ -39,7 +40,7 @@
 namespace pj {
 
 constexpr unsigned long long kHashEmpty = ~0ull;
-constexpr int kDsStack = 192;     // traversal stack entries per thread
+constexpr int kDsStack = 192;     // plain depth-first order's stack entries
 constexpr int kParList = 48;      // objects a parity ray tracks
 constexpr int kHashProbes = 2048;  // probes before a hashmap counts as full
 
@@ -47,10 +48,6 @@ enum { DS_EDGES = 0, DS_NODES, DS_TRIS, DS_HITS, DS_RAYS, DS_OVERFLOW, DS_ERR, D
        DS_NOBJ, DS_FULL, DS_NSTAT };
 
 struct DsSide {
-  const float *xyz;
-  const int32_t *tris;
-  const uint8_t *emask;
-  const int64_t *toff;
   int64_t M, F;
   const float4 *mrec;    // per mesh: box, first lexicographic vertex
   const float *aabb;     // per mesh: closed box
@@ -139,10 +136,11 @@ __device__ __forceinline__ void flush_stats(unsigned long long *st, const unsign
 // once for all of them: the children of up to 32 / W nodes, one to a lane, are
 // tested against the box around the packet, and each that meets it against
 // every lane's triangle; a part of T that no lane meets is never entered.
-// Where a child is smaller than the triangle, its owned edges are tested too (a vessel's triangle is larger than most of a nucleus: by boxes alone
-// it met thousands of leaves that its edges pass by).  A leaf and a lane that
-// meet are listed in shared memory and the list is worked off a pair to a
-// lane: box tests, then the exact test.
+// Where a child is smaller than the triangle, its owned edges are tested too
+// (a vessel's triangle is larger than most of a nucleus: by boxes alone it met
+// thousands of leaves that its edges pass by).  A leaf and a lane that meet
+// are listed in shared memory and the list is worked off a pair to a lane: box
+// tests, then the exact test.
 //
 // Boxes are compared open: a strict crossing has strictly overlapping boxes
 // on every axis (an edge and a triangle whose boxes only touch meet at an
@@ -384,9 +382,13 @@ __global__ void __launch_bounds__(32 * kDsWarps, 4) k_ds_edges(DsSide A, DsSide 
 // (k_ds_edges) took 2.0 M node visits and 1,100 us; 190 now.
 //
 // The walk is breadth first, a launch per level, the narrow ones in one block.
-// What bounds it is each level's launch and chain of dependent reads.  Queue and list are of fixed size; where they do not
-// suffice (DS_FULL: dense data) the packets trace the edges after all, as they
-// do for a self join, in which every triangle meets its own mesh's.
+// What bounds it is each level's launch and chain of dependent reads.  Queues
+// and list are of fixed size, 10,000 x 500 tissue meshes put 3.9 M entries in
+// all through them; where they do not suffice (DS_FULL: dense data) the packets
+// trace the edges after all, as they do for a self join, in which every
+// triangle meets its own mesh's (16 x 16 spheres of 20,480 triangles crossing
+// each other: 6.0 ms of tracing with the walk that is given up, 28 for an edge
+// per thread).
 // ---------------------------------------------------------------------------
 constexpr uint32_t kDsOpen = 0x40000000u;   // the item's children are taken
 constexpr uint32_t kDsIdx = 0x3FFFFFFFu;    // node, or node * W + k of a leaf
@@ -888,10 +890,6 @@ static pj_status dataset_bvh(Ctx *ctx, Dataset *ds, int W, int L, cudaStream_t s
 
 static DsSide ds_side(Dataset *d, Bvh *b) {
   DsSide x;
-  x.xyz = d->d_xyz;
-  x.tris = d->d_tris;
-  x.emask = d->d_emask;
-  x.toff = d->d_toff;
   x.M = d->M;
   x.F = d->F;
   x.mrec = d->d_mrec;
@@ -974,7 +972,10 @@ pj_status run_dataset_join(Ctx *ctx, Dataset *A, Dataset *B, int self_join,
     if (q0) q1 = (uint2 *)ws_get(ctx, "ds_queue1", sizeof(uint2) * (size_t)kDsQueue, &st);
     if (q1) leaves = (uint2 *)ws_get(ctx, "ds_leaves", sizeof(uint2) * (size_t)kDsLeaves, &st);
     if (leaves) lv_cnt = (unsigned *)ws_get(ctx, "ds_levels", 4 * (2 * kDsLevels + 1), &st);
-    if (!lv_cnt) dual = false;  // no room for the walk's 136 MB: the packets need none
+    if (!lv_cnt) {  // no room for the walk's 168 MB: the packets need none
+      dual = false;
+      clear_err(ctx);
+    }
   }
   // one tracing pass over every item: the warps that test the leaf pairs, or
   // A's packets of triangles and B's; B's objects, A's objects (count / emit

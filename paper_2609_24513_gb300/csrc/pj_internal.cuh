@@ -118,8 +118,12 @@ struct Exec {
 };
 
 constexpr size_t kExecBytes = 128;
-// pairs of a host result that come back with the counts
+// pairs of a host result that come back with the counts, and of a device
+// result: its buffer, taken before the pairs' number is known, is held as long
+// as the caller holds the result (16 KB; the 10,000 x 500 tissue join has 1,752
+// pairs).  Larger results are copied once the number is known.
 constexpr int64_t kFirstPairs = 32768;
+constexpr int64_t kFirstDevicePairs = 2048;
 
 struct Serve;  // serving state (pj_serve.cu)
 

@@ -1838,9 +1838,8 @@ __global__ void k_pred_combine(uint8_t *flags, const uint8_t *pflags, const int6
 // pairs with 2 lanes per task (4 at W = 8); a leaf round reads the triangles
 // of 16 / L leaf pairs into registers, 2 L lanes to a pair, filters (edge,
 // triangle) tests by boxes and runs the exact tests that remain one per lane.
-// A round
-// thus waits for one memory latency however many fetches it makes.  A warp
-// takes new candidates whenever its stack holds less than one round.
+// A round thus waits for one memory latency however many fetches it makes.  A
+// warp takes new candidates whenever its stack holds less than one round.
 //
 // Intake.  How many it takes follows what they cost: 8 at first (or an equal
 // share of the candidates, if that is less), four times as many (up to 32) when
@@ -1866,13 +1865,14 @@ __global__ void k_pred_combine(uint8_t *flags, const uint8_t *pflags, const int6
 // a half and three quarters of a warp per SM the urban join took 800, 727,
 // 570 and 541 us, the instanced pairs 1,120, 1,105, 945 and 926) gives the
 // older half of its stack (the larger subtrees) to the queue, and so does a
-// warp whose stack is nearly full.  A costly pair thus spreads over more and more warps.  At most
-// `hungry_max` warps wait for tasks (a warp that finds that many waiting
-// leaves): a heavy pair needs tens of helpers, not thousands of warps
-// polling the same words (a cap of 6 per SM; with 2 per SM 4,429 x 260
-// tissue within at W = 8 took 270 us, with 4 252; 200 x 200 spheres took 200
-// us with 4, 181 with 6; the others the same).  A crossing sets the candidate's flag; the tasks
-// of a flagged candidate are dropped when popped or claimed.
+// warp whose stack is nearly full.  A costly pair thus spreads over more and
+// more warps.  At most `hungry_max` warps wait for tasks (a warp that finds
+// that many waiting leaves): a heavy pair needs tens of helpers, not thousands
+// of warps polling the same words (a cap of 6 per SM; with 2 per SM 4,429 x
+// 260 tissue within at W = 8 took 270 us, with 4 252; 200 x 200 spheres took
+// 200 us with 4, 181 with 6; the others the same).  A crossing sets the
+// candidate's flag; the tasks of a flagged candidate are dropped when popped
+// or claimed.
 //
 // Queue protocol.  Entries are uint4 (candidate, item A, item B, ready).  A
 // producer reserves slots with an atomic add on `tail`, writes the first
@@ -2467,8 +2467,8 @@ __global__ void __launch_bounds__(128, 4) k_stream(StreamArgs P) {
     // one lane per (task, side) copies the W child slots of an expanding
     // node, or the one slot of the item's own box.  (Spreading a node's
     // pieces over consecutive lanes, so that each copy request is one
-    // coalesced run, measured slower here: 0.281 against 0.265 ms on the
-    // pathology step; the leaf triangles below do gain from it.)
+    // coalesced run, measured slower: 0.281 against 0.265 ms on the pathology
+    // step.)
     for (int is = lane; is < npop * 2; is += 32) {
       const int side = is & 1, i = is >> 1;
       const uint4 e = stk[sp - 1 - i];
@@ -3758,8 +3758,8 @@ pj_status run_join(Ctx *ctx, Dataset *A, Dataset *B, const int32_t *cand,
     ~Result() { drop(); }
   } first{ctx};
   const bool borrow = cur_exec(ctx)->borrow_out;
-  const int64_t first_cap =
-      std::min<int64_t>(std::max<int64_t>(Ccap, 1), o->out_host ? kFirstPairs : 2048);
+  const int64_t first_cap = std::min<int64_t>(
+      std::max<int64_t>(Ccap, 1), o->out_host ? kFirstPairs : kFirstDevicePairs);
   int32_t *h_first = reinterpret_cast<int32_t *>((char *)cur_exec(ctx)->h_pinned + 4096);
   if (!borrow && o->out_host) {
     PJ_CK(cudaMemcpyAsync(h_first, d_pairs, 8 * (size_t)first_cap, cudaMemcpyDeviceToHost, s));
@@ -3883,7 +3883,7 @@ pj_status run_join(Ctx *ctx, Dataset *A, Dataset *B, const int32_t *cand,
 //
 // The refinement is the streaming kernel's.  A warp per pair in plain
 // depth-first order, one task a step, left the costliest pair to one warp:
-// 1,501 x 75 tissue meshes took 2,200-7,200 us by seed, 121 us now.
+// 1,501 x 75 tissue meshes took 2,200-7,200 us by seed, 100 us now.
 // ---------------------------------------------------------------------------
 constexpr int64_t kNoAllocMaxChunks = 4096;
 constexpr int64_t kNoAllocMaxCand = kNoAllocMaxChunks * CMP_CHUNK;  // 16,777,216
